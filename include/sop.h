@@ -72,10 +72,10 @@ typedef enum {
  *                              result was computed from part of its input
  *                              (the surrogate's near-field search found
  *                              more than 4,096 centres within r_near);
- *   SOP_DEVSTAT_TIMEOUT        a kernel's bounded wait for the tensor cores
- *                              (the surrogate network's completion
- *                              barrier) gave up; that launch's outputs are
- *                              not valid;
+ *   SOP_DEVSTAT_TIMEOUT        a kernel's bounded wait (the surrogate
+ *                              network's completion barrier, the exchange
+ *                              between the CTAs of the probe placement)
+ *                              gave up; that launch's outputs are not valid;
  *   SOP_DEVSTAT_GRID_COARSENED information, not an error: the bake's
  *                              binning grid was coarsened on the device
  *                              until the cell lists fit the workspace.
@@ -668,9 +668,9 @@ size_t sop_place_probes_workspace_bytes(int64_t n_points);
  * and the same on every run. out_idx [k] (int64, device): the chosen
  * points in order; out_pos [k][3] (device, or NULL): pts + offset nrm,
  * computed in double and rounded once (nrm [n][3] device, or NULL: no
- * offset). 1 <= k <= n, 0 <= start < n. Runs as one thread-block cluster
- * (16 CTAs where the device holds such a cluster, else 8) for all k
- * iterations. Asynchronous. */
+ * offset). 1 <= k <= n, 0 <= start < n. Runs as one cooperative launch for
+ * all k choices, with one CTA an SM (one CTA for at most 2,048 points).
+ * Asynchronous. */
 sop_status sop_place_probes(const float* pts, const float* nrm, int64_t n_points, int32_t k, int64_t start,
                             float offset, int64_t* out_idx, float* out_pos, void* ws, size_t ws_bytes, void* stream);
 

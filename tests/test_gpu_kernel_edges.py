@@ -20,6 +20,27 @@ def cuda(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
+@pytest.mark.parametrize("n,k,scale", [
+    (2, 2, 1.0), (513, 100, 1.0),                    # one CTA
+    (4096, 300, 1.0), (4097, 300, 1.0),              # one CTA / several
+    (155_648, 40, 1.0), (155_649, 40, 1.0),          # 2 / 4 points a thread on 152 SMs
+    (311_297, 40, 1.0), (622_593, 40, 1.0),          # 8, 10
+    (778_241, 30, 1.0), (1_245_185, 30, 1.0),        # 16, keys in the workspace
+    (5000, 50, 1500.0), (1_300_000, 20, 1500.0),     # differences beyond 2^31 quantised units
+])
+def test_fps_point_counts(sop, orc, n, k, scale):
+    """Whole-number results: the indices equal the oracle's at every split of
+    the points over threads and CTAs."""
+    rng = np.random.default_rng(n)
+    pts = (rng.uniform(-1, 1, (n, 3)) * scale).astype(F)
+    pts[n // 3: n // 3 + 20] = pts[0]  # equal points: ties, keys of zero
+    start = n - 1
+    idx, pos = sop.place_probes(cuda(pts), k, start=start)
+    oi, _ = orc.fps(pts, k, start=start)
+    assert np.array_equal(idx.cpu().numpy(), oi)
+    assert np.array_equal(pos.cpu().numpy(), pts[oi])
+
+
 @pytest.mark.parametrize("H,S", [(2, 1), (3, 7), (45, 33), (46, 4096), (91, 64), (512, 9)])
 @pytest.mark.parametrize("values", ["lognormal", "wide", "flat", "zero", "one"])
 def test_importance_texels(sop, orc, H, S, values):
