@@ -56,3 +56,64 @@ def test_importance_texels(sop, orc, H, S, values):
     want = orc.env_importance_dirs(env, S)
     assert np.max(np.abs(got[:, :3] - want[:, :3])) < 2e-7  # one float32 rounding of a unit vector
     np.testing.assert_allclose(got[:, 3], want[:, 3], rtol=2e-7)
+
+
+def _query_workload(P, R, M, He, seed):
+    """Points above a bumpy sheet of probes, iid maps, a smooth environment
+    (so that FP32 direction rounding stays far below the tolerance)."""
+    rng = np.random.default_rng(seed)
+    pp = np.concatenate([rng.uniform(-1, 1, (P, 2)), 0.1 * rng.standard_normal((P, 1))], axis=1).astype(F)
+    x = np.concatenate([rng.uniform(-1.2, 1.2, (M, 2)), 0.1 * rng.standard_normal((M, 1))], axis=1).astype(F)
+    n = rng.standard_normal((M, 3))
+    wo = rng.standard_normal((M, 3))
+    wo *= np.sign(np.sum(wo * n, axis=1, keepdims=True))  # seen from above the surface
+    n, wo = (v / np.linalg.norm(v, axis=1, keepdims=True) for v in (n, wo))
+    th = (np.arange(He) + 0.5) / He * np.pi
+    ph = (np.arange(2 * He) + 0.5) / He * np.pi
+    env = (1.0 + 0.5 * np.sin(th)[:, None, None] * np.cos(ph[None, :, None] + np.arange(3))).astype(F)
+    return dict(pp=pp, x=x, n=n.astype(F), wo=wo.astype(F), albedo=rng.uniform(0, 1, (M, 3)).astype(F),
+                rough=rng.uniform(0.3, 1, M).astype(F), metal=rng.uniform(0, 1, M).astype(F), env=env,
+                rgb=rng.uniform(0, 0.5, (P, R, R, 3)).astype(F), occ=rng.uniform(0, 1, (P, R, R)).astype(F))
+
+
+PTS = ("x", "n", "wo", "albedo", "rough", "metal")
+
+
+@pytest.mark.parametrize("M,P,R,K,S", [
+    (1, 8, 2, 8, 5), (7, 40, 3, 1, 33), (9, 40, 16, 8, 128), (64, 64, 16, 8, 100), (333, 200, 16, 4, 129),
+    (65, 100, 11, 16, 64), (33, 100, 8, 32, 96), (40, 50, 24, 8, 256), (5, 8, 64, 4, 40),
+])
+@pytest.mark.parametrize("caller_dirs", [False, True])
+def test_shade_and_adjoint_shapes(sop, orc, M, P, R, K, S, caller_dirs):
+    """SHADE and its adjoint over remainders of the warp (32 directions) and
+    of the eight points of a CTA, one to 32 probes, maps from 2x2 to 64x64,
+    the library's directions or the caller's. Tolerances as for the oracle
+    tests of either: 1e-5 of the output plus its sensitivity to 2e-6 rad;
+    gradients 1e-4 plus 2e-4 of the terms' magnitudes."""
+    c = _query_workload(P, R, M, 16, 100 * M + R)
+    rng = np.random.default_rng(S)
+    dirs = None
+    if caller_dirs:
+        d = rng.standard_normal((S, 3))
+        d[:, 2] = np.abs(d[:, 2]) + 0.2
+        dirs = (d / np.linalg.norm(d, axis=1, keepdims=True)).astype(F)
+    at = sop.make_atlas(cuda(c["pp"]), R, with_depth=False)
+    sop.atlas_pack(cuda(c["rgb"]), cuda(c["occ"]), None, at)
+    pts = [cuda(c[k]) for k in PTS]
+    gd = None if dirs is None else cuda(dirs)
+    out = sop.query_shade(*pts, at, cuda(c["env"]), K, S, dirs_local=gd).cpu().numpy()
+    args = [c[k] for k in PTS] + [c["pp"], c["rgb"], c["occ"], c["env"], K, S]
+    kw = dict(dirs=None if dirs is None else dirs.astype(np.float64))
+    want, _, _ = orc.query_shade(*args, **kw)
+    sens = orc.query_shade_sensitivity(*args, **kw)
+    assert np.all(np.abs(out - want) <= 1e-5 * np.maximum(np.abs(want), 1e-3 * np.abs(want).mean()) + sens)
+    go = rng.standard_normal((M, 3)).astype(F)
+    g = sop.query_shade_backward(*pts, at, cuda(c["env"]), K, S, cuda(go), dirs_local=gd)
+    w = orc.query_shade_grad(*args, go, **kw)
+    for key in ("albedo", "rough", "metal", "normal"):
+        d = np.abs(g[key].cpu().numpy() - w[key])
+        terms = w["abs_" + key][:, None] if key == "normal" else w["abs_" + key]
+        assert np.all(d <= 1e-4 * np.abs(w[key]) + 2e-4 * terms + 1e-12), key
+    for got, ref in ((g["env"], w["env"]), (g["maps"][..., :3], w["maps_rgb"]), (g["maps"][..., 3], w["maps_occ"])):
+        d = np.abs(got.cpu().numpy() - ref)
+        assert np.all(d <= 1e-4 * np.abs(ref) + 2e-5 * np.abs(ref).max() + 1e-12)
