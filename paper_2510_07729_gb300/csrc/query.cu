@@ -1,21 +1,18 @@
 // SOP query + shade (Sec. 3.1.2 Eq. 2-6, Sec. 3.2.2 Eq. 7-9) for sm_103a.
 //
-// Kernels, in launch order:
-//   probe_grid_kernel   one CTA: quantise probe positions to 2^-20, counting
-//                       sort into a uniform grid of ~P cells;
-//   knn_kernel          one thread per point: exact K nearest probes by
-//                       integer squared distance (ring search with an exact
-//                       integer stopping bound), then the Eq. 4-6 weights;
-//   env_pack_kernel     environment to float4 with a wrapped column and
-//                       clamped rows so the bilinear fetch needs no branches;
-//   atlas_quad_kernel   bilinear footprints of the atlas (RGBO, SHADE mode)
-//   / atlas_occ_quad_*  or occlusion alone (SHADOW mode reads only O);
-//   dirs_kernel         local light directions (Hammersley in fp64 -> fp32);
-//   shade_kernel        LANES threads per point split the S directions; per
-//                       direction one octahedral encode (world-frame maps),
-//                       4 texel fetches per probe from the L2-resident atlas,
-//                       environment bilinear, BRDF, fp32 accumulation, and a
-//                       shuffle reduction over the point's lanes.
+// Launches of a query, in order:
+//   query_tables_kernel  the probe grid (one CTA) beside the tables: light
+//                        directions (Hammersley in fp64 -> fp32), bilinear
+//                        footprints of the environment and of the atlas;
+//   knn_warp_kernel /    exact K nearest probes by integer squared distance
+//   knn_kernel           (rings of grid cells with an exact integer stopping
+//                        bound), then the Eq. 4-6 weights; a warp or a
+//                        thread a point;
+//   one of               shade_kernel (LANES threads a point split the S
+//                        directions, 4 texel fetches per probe and direction
+//                        from the L2-resident footprints), shade_point_kernel
+//                        (a warp a point, probes blended first),
+//                        shade_world_kernel (importance-sampled directions).
 #include <float.h>
 #include <stdlib.h>
 
@@ -41,7 +38,6 @@ QueryLayout query_layout(int32_t P, int64_t M, int32_t K, int32_t S, int32_t He,
     L.cell_start = o; o = align256(o + sizeof(int32_t) * (size_t)(L.cells_cap + 1));
     L.cell_cnt = o;   o = align256(o + sizeof(int32_t) * (size_t)L.cells_cap);
     L.entries = o;    o = align256(o + sizeof(int4) * (size_t)P);
-    L.env4 = o;       o = align256(o + sizeof(float4) * (size_t)(He + 2) * (We + 1));
     L.envq = o;       o = align256(o + 64 * (size_t)(He + 1) * (We + 1));  // both layouts
     L.quads = o;      o = align256(o + (rgbo_dtype == SOP_F32 ? 64 : 32) * (size_t)P * (R + 1) * (R + 1));
     L.dirs = o;       o = align256(o + sizeof(float4) * (size_t)S);
@@ -87,31 +83,76 @@ __device__ __forceinline__ int64_t grid_cell_edge(const int64_t ext[3], int64_t 
     return lo;
 }
 
-// ---------------------------------------------------------------------------
-// Probe grid (single CTA; P is small: thousands to ~1e5 probes).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) probe_grid_kernel(const float* __restrict__ probe_pos, int32_t P, int32_t g_axis,
-                                                           ProbeGrid* grid, int32_t* cell_start, int32_t* cell_cnt,
-                                                           int4* entries)
+// cell of a site of the set (quantised position), by the grid's edge
+__device__ __forceinline__ int grid_cell(const ProbeGrid& G, int32_t qx, int32_t qy, int32_t qz)
 {
-    __shared__ int32_t s_min[3], s_max[3];
-    __shared__ int32_t s_part[1024];
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const uint32_t cs = (uint32_t)G.cs;
+    const int cx = (int)div_by((uint32_t)qx - (uint32_t)G.qmin[0], cs, G.inv);
+    const int cy = (int)div_by((uint32_t)qy - (uint32_t)G.qmin[1], cs, G.inv);
+    const int cz = (int)div_by((uint32_t)qz - (uint32_t)G.qmin[2], cs, G.inv);
+    return (cz * G.dims[1] + cy) * G.dims[0] + cx;
+}
+
+// ---------------------------------------------------------------------------
+// Probe grid, built by one CTA of 1,024 threads (P is small: thousands to
+// ~1e5 probes). A serial chain of short steps, so each is kept short: the
+// candidate edges of all five coarsening levels are searched at once, a warp
+// each, 32 edges a step; cells are counted, scanned and filled in shared
+// memory while they fit (kGridSmemCells); divisions by the edge are one
+// multiplication. 4,096 probes: 26-49 us when one thread bisected each edge
+// by 64-bit divisions and the cells were counted in memory; with all of a
+// query's tables beside it 16-20 us now.
+// ---------------------------------------------------------------------------
+constexpr int kGridThreads = 1024;
+constexpr int kGridLevels = 5;
+constexpr int kGridSmemCells = 8192;
+
+struct GridSmem {
+    int32_t mn[3], mx[3];
+    uint32_t edge[kGridLevels];
+    int32_t occ;
+    int32_t warp[32];
+    int32_t cnt[kGridSmemCells];
+};
+
+// Cells of edge e over a box of extents ext; at most cap?
+__device__ __forceinline__ bool grid_fits(const uint32_t ext[3], uint64_t e, int64_t cap)
+{
+    uint64_t n = 1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        n *= (e > ext[a] ? 0u : ext[a] / (uint32_t)e) + 1u;
+        if (n > (uint64_t)cap) return false;
+    }
+    return true;
+}
+
+__device__ __forceinline__ void probe_grid_build(GridSmem& sm, const float* __restrict__ probe_pos, int32_t P,
+                                                 int32_t g_axis, ProbeGrid* grid, int32_t* cell_start,
+                                                 int32_t* cell_cnt, int4* entries)
+{
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, nt = kGridThreads, lane = tid & 31, warp = tid >> 5;
     if (tid < 3) {
-        s_min[tid] = INT32_MAX;
-        s_max[tid] = INT32_MIN;
+        sm.mn[tid] = INT32_MAX;
+        sm.mx[tid] = INT32_MIN;
     }
     __syncthreads();
     int32_t lmin[3] = {INT32_MAX, INT32_MAX, INT32_MAX}, lmax[3] = {INT32_MIN, INT32_MIN, INT32_MIN};
     for (int p = tid; p < P; p += nt)
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            int32_t q = quantise(probe_pos[3 * p + a]);
+            const int32_t q = quantise(probe_pos[3 * p + a]);
             lmin[a] = min(lmin[a], q);
             lmax[a] = max(lmax[a], q);
         }
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        atomicMin(&s_min[a], lmin[a]);
-        atomicMax(&s_max[a], lmax[a]);
+        const int32_t lo = __reduce_min_sync(full, lmin[a]), hi = __reduce_max_sync(full, lmax[a]);
+        if (lane == 0 && lo <= hi) {
+            atomicMin(&sm.mn[a], lo);
+            atomicMax(&sm.mx[a], hi);
+        }
     }
     __syncthreads();
     // cell edge: the finest grid within (g+1)^3 cells, coarsened (cap
@@ -119,78 +160,114 @@ __global__ void __launch_bounds__(1024) probe_grid_kernel(const float* __restric
     // occupied cell. A volume-like set keeps the fine grid; a flat one (the
     // shadow probes on the ground), whose far query points need the K
     // nearest from a wide strip, gets cells of a few probes each.
-    __shared__ ProbeGrid G;
-    __shared__ int64_t s_cap;
-    __shared__ int32_t s_occ;
-    if (tid == 0) s_cap = (int64_t)(g_axis + 1) * (g_axis + 1) * (g_axis + 1);
-    for (int it = 0;; ++it) {
-        if (tid == 0) {
-            int64_t ext[3];
-            for (int a = 0; a < 3; ++a) ext[a] = (int64_t)s_max[a] - s_min[a];
-            const int64_t cs = grid_cell_edge(ext, s_cap);
-            G.cs = (int32_t)cs;
-            int32_t nc = 1;
-            for (int a = 0; a < 3; ++a) {
-                G.qmin[a] = s_min[a];
-                G.dims[a] = (int32_t)(ext[a] / cs) + 1;
-                nc *= G.dims[a];
+    const int64_t cap0 = (int64_t)(g_axis + 1) * (g_axis + 1) * (g_axis + 1);
+    uint32_t ext[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) ext[a] = (uint32_t)sm.mx[a] - (uint32_t)sm.mn[a];
+    if (warp < kGridLevels) {
+        // smallest edge that fits, 32 candidates a step
+        const int64_t cap = cap0 >> warp;
+        uint64_t lo = 1, hi = (uint64_t)max(ext[0], max(ext[1], ext[2])) + 1;  // hi: one cell per axis
+        while (lo < hi) {
+            const uint64_t step = (hi - lo + 31) / 32, e = min(lo + lane * step, hi);
+            const unsigned ok = __ballot_sync(full, grid_fits(ext, e, cap));
+            const int f = ok ? __ffs(ok) - 1 : 32;
+            if (f == 0) hi = lo;
+            else {
+                if (f < 32) hi = min(lo + f * step, hi);
+                lo = min(lo + (f - 1) * step, hi) + 1;
             }
-            G.ncells = nc;
-            s_occ = 0;
         }
-        __syncthreads();
-        for (int c = tid; c < G.ncells; c += nt) cell_cnt[c] = 0;
-        __syncthreads();
-        for (int p = tid; p < P; p += nt) {
-            int c[3];
-            for (int a = 0; a < 3; ++a) c[a] = (int)(((int64_t)quantise(probe_pos[3 * p + a]) - G.qmin[a]) / G.cs);
-            if (atomicAdd(&cell_cnt[(c[2] * G.dims[1] + c[1]) * G.dims[0] + c[0]], 1) == 0) atomicAdd(&s_occ, 1);
+        // (an edge of 2^32 - 1 and more: one cell per axis too)
+        if (lane == 0) sm.edge[warp] = (uint32_t)min(lo, (uint64_t)INT32_MAX);
+    }
+    __syncthreads();
+    const bool in_smem = cap0 <= kGridSmemCells;
+    int32_t* cnt = in_smem ? sm.cnt : cell_cnt;
+    ProbeGrid G;
+    for (int it = 0;; ++it) {
+        const uint32_t cs = sm.edge[it];
+        G.cs = (int32_t)cs;
+        G.inv = 0xffffffffu / cs;
+        G.ncells = 1;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            G.qmin[a] = sm.mn[a];
+            G.dims[a] = (int32_t)(ext[a] / cs) + 1;
+            G.ncells *= G.dims[a];
         }
+        if (tid == 0) sm.occ = 0;
+        for (int c = tid; c < G.ncells; c += nt) cnt[c] = 0;
         __syncthreads();
-        const bool again = it < 4 && (int64_t)P < 3 * (int64_t)s_occ && s_cap > 8;
+        int occ = 0;
+        for (int p = tid; p < P; p += nt)
+            if (atomicAdd(&cnt[grid_cell(G, quantise(probe_pos[3 * p]), quantise(probe_pos[3 * p + 1]),
+                                         quantise(probe_pos[3 * p + 2]))], 1) == 0)
+                ++occ;
+        occ = __reduce_add_sync(full, occ);
+        if (lane == 0 && occ) atomicAdd(&sm.occ, occ);
+        __syncthreads();
+        const bool again = it < kGridLevels - 1 && (int64_t)P < 3 * (int64_t)sm.occ && (cap0 >> it) > 8;
         __syncthreads();
         if (!again) break;
-        if (tid == 0) s_cap >>= 1;
     }
     if (tid == 0) *grid = G;
-    const int nc = G.ncells;
-    // exclusive scan of cell counts: contiguous chunk per thread + block scan
-    const int chunk = (nc + nt - 1) / nt;
-    const int c0 = tid * chunk, c1 = min(nc, c0 + chunk);
+    // exclusive scan of the counts: a contiguous chunk per thread, then the block
+    const int nc = G.ncells, chunk = (nc + nt - 1) / nt;
+    const int c0 = min(nc, tid * chunk), c1 = min(nc, c0 + chunk);
     int32_t sum = 0;
-    for (int c = c0; c < c1; ++c) sum += cell_cnt[c];
-    s_part[tid] = sum;
+    for (int c = c0; c < c1; ++c) sum += cnt[c];
+    int32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t v = __shfl_up_sync(full, inc, o);
+        if (lane >= o) inc += v;
+    }
+    if (lane == 31) sm.warp[warp] = inc;
     __syncthreads();
-    for (int off = 1; off < nt; off <<= 1) {
-        int32_t v = (tid >= off) ? s_part[tid - off] : 0;
-        __syncthreads();
-        s_part[tid] += v;
-        __syncthreads();
+    if (warp == 0) {
+        const int32_t w = sm.warp[lane];
+        int32_t v = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t u = __shfl_up_sync(full, v, o);
+            if (lane >= o) v += u;
+        }
+        sm.warp[lane] = v - w;
     }
-    int32_t run = s_part[tid] - sum;
+    __syncthreads();
+    int32_t run = inc - sum + sm.warp[warp];
     for (int c = c0; c < c1; ++c) {
-        int32_t v = cell_cnt[c];
+        const int32_t v = cnt[c];
         cell_start[c] = run;
+        cnt[c] = in_smem ? run : 0;  // the fill's cursor
         run += v;
-        cell_cnt[c] = 0;
     }
-    if (tid == nt - 1) cell_start[nc] = s_part[nt - 1];
+    if (tid == nt - 1) cell_start[nc] = P;
     __syncthreads();
     for (int p = tid; p < P; p += nt) {
-        int32_t q[3];
-        int c[3];
-        for (int a = 0; a < 3; ++a) {
-            q[a] = quantise(probe_pos[3 * p + a]);
-            c[a] = (int)(((int64_t)q[a] - G.qmin[a]) / G.cs);
-        }
-        int cell = (c[2] * G.dims[1] + c[1]) * G.dims[0] + c[0];
-        int pos = cell_start[cell] + atomicAdd(&cell_cnt[cell], 1);
-        entries[pos] = make_int4(q[0], q[1], q[2], p);
+        const int32_t qx = quantise(probe_pos[3 * p]), qy = quantise(probe_pos[3 * p + 1]),
+                      qz = quantise(probe_pos[3 * p + 2]);
+        const int cell = grid_cell(G, qx, qy, qz);
+        const int at = atomicAdd(&cnt[cell], 1) + (in_smem ? 0 : cell_start[cell]);
+        entries[at] = make_int4(qx, qy, qz, p);
     }
 }
 
-// floor division for possibly negative numerators (positive divisor)
-__device__ __forceinline__ int64_t floordiv(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
+__global__ void __launch_bounds__(kGridThreads) probe_grid_kernel(const float* __restrict__ probe_pos, int32_t P,
+                                                                  int32_t g_axis, ProbeGrid* grid, int32_t* cell_start,
+                                                                  int32_t* cell_cnt, int4* entries)
+{
+    __shared__ GridSmem sm;
+    probe_grid_build(sm, probe_pos, P, g_axis, grid, cell_start, cell_cnt, entries);
+}
+
+// the point's cell along one axis, clamped into the grid
+__device__ __forceinline__ int grid_axis_cell(const ProbeGrid& G, int a, int32_t q)
+{
+    if (q < G.qmin[a]) return 0;
+    return min((int)div_by((uint32_t)q - (uint32_t)G.qmin[a], (uint32_t)G.cs, G.inv), G.dims[a] - 1);
+}
 
 // The search visits rings of cells (Chebyshev radius r in cell indices)
 // around cc, the point's cell clamped into the grid. This is a lower bound on
@@ -217,8 +294,8 @@ __device__ __forceinline__ uint64_t unsearched_bound2(const ProbeGrid& G, const 
         const uint64_t rest = osum - out2[b];
         // d^2 + rest, unless it exceeds 64 bits (then it bounds nothing)
         auto take = [&](uint64_t d) {
-            if (__umul64hi(d, d) != 0) return;
-            const uint64_t v = d * d + rest;
+            if (d >> 32) return;
+            const uint64_t v = (uint64_t)(uint32_t)d * (uint32_t)d + rest;
             if (v >= rest && v < best) best = v;
         };
         // cells of index <= cc_b - r - 1 end at qmin + (cc_b - r) cs
@@ -256,11 +333,7 @@ __global__ void __launch_bounds__(128, KMAX <= 8 ? 8 : 1) knn_kernel(const float
     }
     const int32_t q[3] = {quantise(xp.x), quantise(xp.y), quantise(xp.z)};
     // rings are taken around the point's cell clamped into the grid
-    int c[3];
-    for (int a = 0; a < 3; ++a) {
-        const int64_t ca = floordiv((int64_t)q[a] - G.qmin[a], G.cs);
-        c[a] = (int)(ca < 0 ? 0 : (ca > G.dims[a] - 1 ? G.dims[a] - 1 : ca));
-    }
+    const int c[3] = {grid_axis_cell(G, 0, q[0]), grid_axis_cell(G, 1, q[1]), grid_axis_cell(G, 2, q[2])};
     uint64_t bk[KMAX];
     int32_t bi[KMAX];
 #pragma unroll
@@ -349,33 +422,196 @@ __global__ void __launch_bounds__(128, KMAX <= 8 ? 8 : 1) knn_kernel(const float
 }
 
 // ---------------------------------------------------------------------------
-// Environment table: float4 [(He+2)][(We+1)], stored row r+1 = row r (rows 0
-// and He+1 repeat the first and last row: v clamps), stored column We =
-// column 0 (u wraps).
+// The same search, one warp per point, for calls that do not fill the machine
+// with a thread a point: a thread's search is a chain of dependent loads
+// (cell, entries, insertion) of 20 to 60 us however few points there are. The
+// lanes take the cells of the cube around the point, 32 at a time, and their
+// entries side by side; candidates gather in shared memory and the K best are
+// picked by warp minima. With few probes (entries NULL) the lanes take all of
+// them and no grid is needed.
 // ---------------------------------------------------------------------------
-__global__ void env_pack_kernel(const float* __restrict__ env, int32_t He, int32_t We, float4* __restrict__ env4,
-                                unsigned int* status)
+constexpr int kKnnWarps = 8;
+constexpr int kKnnBuf = 128;  // candidates a warp holds
+
+struct KnnK {
+    const float *x, *nrm;
+    int64_t M;
+    int32_t K, P;
+    uint64_t snap_key, r2_key;
+    const ProbeGrid* grid;
+    const int32_t* cell_start;
+    const int4* entries;
+    const float* probe_pos;
+    int32_t* ws_idx;
+    float* ws_w;
+    int32_t* user_idx;
+    float* user_w;
+    unsigned int* status;
+};
+
+// The K best of the cnt candidates, sorted, to the front; returns their number.
+__device__ __forceinline__ int knn_select(uint64_t* key, int32_t* id, int cnt, int K, int lane)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n = (int64_t)(He + 2) * (We + 1);
-    if (i >= n) return;
-    const int rs = (int)(i / (We + 1)), cs = (int)(i % (We + 1));
-    const int r = min(max(rs - 1, 0), He - 1), c = cs == We ? 0 : cs;
-    const float* e = env + ((int64_t)r * We + c) * 3;
-    if (!isfinite(e[0] + e[1] + e[2]) && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
-    env4[i] = make_float4(e[0], e[1], e[2], 0.f);
+    constexpr int PER = kKnnBuf / 32;
+    const unsigned full = 0xffffffffu;
+    uint64_t lk[PER];
+    int32_t li[PER];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const bool on = j * 32 + lane < cnt;
+        lk[j] = on ? key[j * 32 + lane] : UINT64_MAX;
+        li[j] = on ? id[j * 32 + lane] : INT32_MAX;
+    }
+    __syncwarp();
+    const int n = min(K, cnt);
+    for (int r = 0; r < n; ++r) {
+        uint64_t bk = lk[0];
+        int32_t bi = li[0];
+#pragma unroll
+        for (int j = 1; j < PER; ++j) {
+            const bool lt = lk[j] < bk || (lk[j] == bk && li[j] < bi);
+            bk = lt ? lk[j] : bk;
+            bi = lt ? li[j] : bi;
+        }
+        const uint32_t hi = __reduce_min_sync(full, (uint32_t)(bk >> 32));
+        const uint32_t lo = __reduce_min_sync(full, (uint32_t)(bk >> 32) == hi ? (uint32_t)bk : 0xffffffffu);
+        const uint64_t wk = (uint64_t)hi << 32 | lo;
+        const int32_t wi = (int32_t)__reduce_min_sync(full, bk == wk ? (uint32_t)bi : (uint32_t)INT32_MAX);
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            if (lk[j] == wk && li[j] == wi) {
+                lk[j] = UINT64_MAX;
+                li[j] = INT32_MAX;
+            }
+        if (lane == 0) {
+            key[r] = wk;
+            id[r] = wi;
+        }
+    }
+    __syncwarp();
+    return n;
+}
+
+__global__ void __launch_bounds__(kKnnWarps * 32) knn_warp_kernel(const KnnK a)
+{
+    __shared__ uint64_t s_key[kKnnWarps][kKnnBuf];
+    __shared__ int32_t s_id[kKnnWarps][kKnnBuf];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t m = (int64_t)blockIdx.x * kKnnWarps + warp;
+    if (m >= a.M) return;
+    uint64_t* key = s_key[warp];
+    int32_t* id = s_id[warp];
+    const int K = a.K;
+    float3 xp = load3(a.x, m);
+    const float3 nr = load3(a.nrm, m);
+    const bool okx = isfinite(xp.x + xp.y + xp.z);
+    if (lane == 0 && (!okx || !isfinite(nr.x + nr.y + nr.z)) && a.status) atomicOr(a.status, SOP_DEVSTAT_NONFINITE);
+    if (!okx) xp = f3(0.f, 0.f, 0.f);
+    const int32_t q[3] = {quantise(xp.x), quantise(xp.y), quantise(xp.z)};
+    int cnt = 0;
+    uint64_t kth = UINT64_MAX;  // no candidate above it can be among the K
+    const auto add = [&](bool on, int4 en) {
+        const uint64_t k = on ? qdist2(en.x, en.y, en.z, q) : UINT64_MAX;
+        const bool pass = on && k <= a.r2_key && k <= kth;
+        const unsigned pm = __ballot_sync(full, pass);
+        if (pass) {
+            const int at = cnt + __popc(pm & ((1u << lane) - 1u));
+            key[at] = k;
+            id[at] = en.w;
+        }
+        cnt += __popc(pm);
+        if (cnt > kKnnBuf - 32) {
+            cnt = knn_select(key, id, cnt, K, lane);
+            kth = cnt == K ? key[K - 1] : UINT64_MAX;
+        }
+    };
+    if (!a.entries) {
+        for (int p0 = 0; p0 < a.P; p0 += 32) {
+            const int p = min(p0 + lane, a.P - 1);
+            add(p0 + lane < a.P, make_int4(quantise(__ldg(a.probe_pos + 3 * p)), quantise(__ldg(a.probe_pos + 3 * p + 1)),
+                                           quantise(__ldg(a.probe_pos + 3 * p + 2)), p));
+        }
+        cnt = knn_select(key, id, cnt, K, lane);
+    } else {
+        const ProbeGrid G = *a.grid;
+        const int c[3] = {grid_axis_cell(G, 0, q[0]), grid_axis_cell(G, 1, q[1]), grid_axis_cell(G, 2, q[2])};
+        // cubes of radius 1, 2, ... cells (each without the one before)
+        for (int r = 1;; ++r) {
+            const int x0 = max(c[0] - r, 0), y0 = max(c[1] - r, 0), z0 = max(c[2] - r, 0);
+            const int nx = min(c[0] + r, G.dims[0] - 1) - x0 + 1, ny = min(c[1] + r, G.dims[1] - 1) - y0 + 1,
+                      nz = min(c[2] + r, G.dims[2] - 1) - z0 + 1, nc = nx * ny * nz;
+            for (int l0 = 0; l0 < nc; l0 += 32) {
+                const int l = l0 + lane;
+                const int xx = x0 + l % nx, yz = l / nx, yy = y0 + yz % ny, zz = z0 + yz / ny;
+                const int far = max(max(abs(xx - c[0]), abs(yy - c[1])), abs(zz - c[2]));
+                int e = 0, e1 = 0;
+                if (l < nc && (r == 1 || far == r)) {
+                    const int cell = (zz * G.dims[1] + yy) * G.dims[0] + xx;
+                    e = __ldg(a.cell_start + cell);
+                    e1 = __ldg(a.cell_start + cell + 1);
+                }
+                while (__any_sync(full, e < e1)) {
+                    const bool on = e < e1;
+                    add(on, on ? __ldg(a.entries + e) : make_int4(0, 0, 0, 0));
+                    ++e;
+                }
+            }
+            cnt = knn_select(key, id, cnt, K, lane);
+            kth = cnt == K ? key[K - 1] : UINT64_MAX;
+            const uint64_t bnd = unsearched_bound2(G, q, c, r);
+            if (bnd == UINT64_MAX || kth < bnd || a.r2_key < bnd) break;
+        }
+    }
+    // weights (Eq. 4-6), lane k for neighbour k; the same arithmetic and order
+    // of the sum as knn_kernel
+    const float nl = sqrtf(dot3(nr, nr));
+    const float3 nn = f3(nr.x / nl, nr.y / nl, nr.z / nl);
+    const bool found = lane < cnt;
+    const int32_t bi = found ? id[lane] : 0;
+    const bool snap = cnt > 0 && key[0] <= a.snap_key;
+    const int32_t fill = cnt > 0 ? id[0] : 0;
+    float w = 0.f;
+    if (found) {
+        const float3 d = load3(a.probe_pos, bi) - xp;
+        const float dl = sqrtf(dot3(d, d));
+        const float ws = 1.f / dl;
+        const float wb = 0.5f * (1.f + dot3(d, nn) / dl) + 0.01f;
+        w = snap ? (lane == 0 ? 1.f : 0.f) : ws * wb;
+    }
+    float wsum = 0.f;
+    for (int k = 0; k < cnt; ++k) wsum += __shfl_sync(full, w, k);
+    if (lane < K) {
+        const float wk = (snap || !found) ? w : w / wsum;
+        a.ws_idx[m * K + lane] = found ? bi : fill;
+        a.ws_w[m * K + lane] = wk;
+        if (a.user_idx) a.user_idx[m * K + lane] = found ? bi : -1;
+        if (a.user_w) a.user_w[m * K + lane] = wk;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Tables of a query, all in one launch with the probe grid (query_tables_kernel):
+// the environment's and the atlas's bilinear footprints, and the directions.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void flag_nonfinite(bool ok, unsigned int* status)
+{
+    if (!ok && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
 }
 
 // Environment footprints: for base (r0, c0), r0 in [0, He], c0 in [0, We),
-// the 2x2 bilinear footprint of the padded table, RGB x 4 = 12 floats in a
-// 64-byte slot: (e00, e01, e10, e11) with e01 = column c0+1, e10 = row r0+1.
-__global__ void env_quad_kernel(const float4* __restrict__ env4, int32_t He, int32_t We, float4* __restrict__ envq)
+// the 2x2 bilinear footprint of rows r0 - 1, r0 (clamped) and columns c0,
+// c0 + 1 (wrapped), RGB x 4 = 12 floats in a 64-byte slot: (e00, e01, e10,
+// e11) with e01 the next column, e10 the next row.
+__device__ __forceinline__ void env_footprint(const float* __restrict__ env, int32_t He, int32_t We, int64_t i,
+                                              float4* __restrict__ envq, unsigned int* status)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)(He + 1) * We) return;
-    const int r0 = (int)(i / We), c0 = (int)(i % We);
-    const float4* p = env4 + (int64_t)r0 * (We + 1) + c0;
-    const float4 a = p[0], b = p[1], c = p[We + 1], d = p[We + 2];
+    const int r0 = (int)(i / We), c0 = (int)(i % We), c1 = c0 + 1 == We ? 0 : c0 + 1;
+    const int ra = max(r0 - 1, 0), rb = min(r0, He - 1);
+    const float3 a = load3(env, (int64_t)ra * We + c0), b = load3(env, (int64_t)ra * We + c1),
+                 c = load3(env, (int64_t)rb * We + c0), d = load3(env, (int64_t)rb * We + c1);
+    flag_nonfinite(isfinite(c.x + c.y + c.z), status);  // (r0 < He covers every texel)
     float4* q = envq + 4 * i;
     q[0] = make_float4(a.x, a.y, a.z, b.x);
     q[1] = make_float4(b.y, b.z, c.x, c.y);
@@ -385,23 +621,20 @@ __global__ void env_quad_kernel(const float4* __restrict__ env4, int32_t He, int
 
 // Octahedral environment footprints (Sec. 4.1 layout, [H][H][3]): for base
 // (a, b) in [0, H]^2, the texels (a-1+di, b-1+dj), di, dj in {0, 1}, through
-// the probe maps' border rule, in the 64-byte slot format of env_quad_kernel
-// (e00, e01 = next column, e10 = next row, e11).
-__global__ void env_oct_quad_kernel(const float* __restrict__ env, int32_t H, float4* __restrict__ envq,
-                                    unsigned int* status)
+// the probe maps' border rule, in the same slots.
+__device__ __forceinline__ void env_oct_footprint(const float* __restrict__ env, int32_t H, int64_t k,
+                                                  float4* __restrict__ envq, unsigned int* status)
 {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int HQ = H + 1;
-    if (k >= (int64_t)HQ * HQ) return;
     const int b = (int)(k / HQ), a = (int)(k % HQ);
     float3 e[4];
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
         int si, sj;
         oct_wrap(H, a - 1 + (q & 1), b - 1 + (q >> 1), si, sj);
-        const float* t = env + ((int64_t)sj * H + si) * 3;
-        e[q] = f3(t[0], t[1], t[2]);
+        e[q] = load3(env, (int64_t)sj * H + si);
     }
-    if (!isfinite(e[0].x + e[0].y + e[0].z) && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
+    flag_nonfinite(isfinite(e[0].x + e[0].y + e[0].z), status);
     float4* o = envq + 4 * k;
     o[0] = make_float4(e[0].x, e[0].y, e[0].z, e[1].x);
     o[1] = make_float4(e[1].y, e[1].z, e[2].x, e[2].y);
@@ -411,77 +644,64 @@ __global__ void env_oct_quad_kernel(const float* __restrict__ env, int32_t H, fl
 
 // Atlas footprints: for probe p and base (a, b) in [0, R]^2 of the stored
 // (gutter) map, the texels (a,b), (a+1,b), (a,b+1), (a+1,b+1) stored
-// contiguously, so one bilinear fetch reads one aligned 32/64-byte block.
+// contiguously, so one bilinear fetch reads one aligned block.
+//   kAtlasQuads: RGBO, 64 or 32 bytes (SHADE);
+//   kAtlasOcc:   O alone, as float4 (float32 atlas) or four 16-bit values
+//                (SHADOW reads only O, Eq. 8);
+//   kAtlasCheck: nothing stored (the kernels that read the atlas itself);
+// in each the texels are checked: every interior texel is the first texel of
+// one footprint.
+enum { kAtlasQuads = 0, kAtlasOcc = 1, kAtlasCheck = 2 };
 template <int DT>
-__global__ void atlas_quad_kernel(const typename Texel<DT>::raw* __restrict__ atlas, int32_t P, int32_t R,
-                                  typename Texel<DT>::raw* __restrict__ quads, unsigned int* status)
+__device__ __forceinline__ void atlas_footprint(const typename Texel<DT>::raw* __restrict__ atlas, int32_t R, int64_t i,
+                                                int what, void* __restrict__ quads, unsigned int* status)
 {
+    using raw = typename Texel<DT>::raw;
     const int RS = R + 2, RQ = R + 1;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)P * RQ * RQ) return;
     const int64_t pr = i / (RQ * RQ);
     const int r = (int)(i % (RQ * RQ));
     const int b = r / RQ, a = r % RQ;
-    const typename Texel<DT>::raw* src = atlas + pr * RS * RS + (int64_t)b * RS + a;
-    typename Texel<DT>::raw* dst = quads + 4 * i;
-    // every interior texel is the first texel of one footprint
-    if (!Texel<DT>::finite(src[0]) && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
-    dst[0] = src[0];
-    dst[1] = src[1];
-    dst[2] = src[RS];
-    dst[3] = src[RS + 1];
-}
-
-// Occlusion footprints for SHADOW mode, which reads only O (Eq. 8): the
-// four O values of each footprint, as float4 (float32 atlas) or four
-// 16-bit values in 8 bytes, so one probe fetch is one 128/64-bit load.
-__global__ void atlas_occ_quad_f32_kernel(const float4* __restrict__ atlas, int32_t P, int32_t R,
-                                          float4* __restrict__ quads, unsigned int* status)
-{
-    const int RS = R + 2, RQ = R + 1;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)P * RQ * RQ) return;
-    const int64_t pr = i / (RQ * RQ);
-    const int r = (int)(i % (RQ * RQ));
-    const int b = r / RQ, a = r % RQ;
-    const float4* src = atlas + pr * RS * RS + (int64_t)b * RS + a;
-    if (!isfinite(src[0].w) && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
-    quads[i] = make_float4(src[0].w, src[1].w, src[RS].w, src[RS + 1].w);
-}
-
-// 16-bit texels (R, G, B, O): O is the upper half of the second word.
-template <int DT>
-__global__ void atlas_occ_quad_16_kernel(const uint2* __restrict__ atlas, int32_t P, int32_t R,
-                                         uint2* __restrict__ quads, unsigned int* status)
-{
-    const int RS = R + 2, RQ = R + 1;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)P * RQ * RQ) return;
-    const int64_t pr = i / (RQ * RQ);
-    const int r = (int)(i % (RQ * RQ));
-    const int b = r / RQ, a = r % RQ;
-    const uint2* src = atlas + pr * RS * RS + (int64_t)b * RS + a;
-    if (!Texel<DT>::finite(src[0]) && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
-    quads[i] = make_uint2((src[0].y >> 16) | (src[1].y & 0xffff0000u), (src[RS].y >> 16) | (src[RS + 1].y & 0xffff0000u));
+    const raw* src = atlas + pr * RS * RS + (int64_t)b * RS + a;
+    const raw t0 = src[0];
+    if (what == kAtlasOcc && DT == SOP_F32) flag_nonfinite(isfinite(reinterpret_cast<const float4&>(t0).w), status);
+    else flag_nonfinite(Texel<DT>::finite(t0), status);
+    if (what == kAtlasCheck) return;
+    const raw t1 = src[1], t2 = src[RS], t3 = src[RS + 1];
+    if (what == kAtlasQuads) {
+        raw* dst = reinterpret_cast<raw*>(quads) + 4 * i;
+        dst[0] = t0;
+        dst[1] = t1;
+        dst[2] = t2;
+        dst[3] = t3;
+    } else if (DT == SOP_F32) {
+        const auto w = [](const raw& t) { return reinterpret_cast<const float4&>(t).w; };
+        reinterpret_cast<float4*>(quads)[i] = make_float4(w(t0), w(t1), w(t2), w(t3));
+    } else {
+        // O is the upper half of the second word
+        const auto y = [](const raw& t) { return reinterpret_cast<const uint2&>(t).y; };
+        reinterpret_cast<uint2*>(quads)[i] = make_uint2((y(t0) >> 16) | (y(t1) & 0xffff0000u),
+                                                        (y(t2) >> 16) | (y(t3) & 0xffff0000u));
+    }
 }
 
 __device__ __forceinline__ double radical_inverse2(uint32_t i) { return (double)__brev(i) * 2.3283064365386963e-10; }
 
-// Local light directions: the caller's set, or the centred Hammersley set.
+// Local light direction i: the caller's, or the centred Hammersley set's.
+__device__ __forceinline__ float3 local_dir(int i, int32_t S, const float* __restrict__ dirs_local)
+{
+    if (dirs_local) return load3(dirs_local, i);
+    const double z = (i + 0.5) / S;
+    const double phi = 6.283185307179586476925 * radical_inverse2((uint32_t)i);
+    const double s = sqrt(1.0 - z * z);
+    return f3((float)(s * cos(phi)), (float)(s * sin(phi)), (float)z);
+}
+
 __global__ void dirs_kernel(int32_t S, const float* __restrict__ dirs_local, float4* __restrict__ out4,
                             float* __restrict__ out3)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S) return;
-    float3 d;
-    if (dirs_local) {
-        d = load3(dirs_local, i);
-    } else {
-        const double z = (i + 0.5) / S;
-        const double phi = 6.283185307179586476925 * radical_inverse2((uint32_t)i);
-        const double s = sqrt(1.0 - z * z);
-        d = f3((float)(s * cos(phi)), (float)(s * sin(phi)), (float)z);
-    }
+    const float3 d = local_dir(i, S, dirs_local);
     if (out4) out4[i] = make_float4(d.x, d.y, d.z, 0.f);
     if (out3) {
         out3[3 * i] = d.x;
@@ -490,13 +710,74 @@ __global__ void dirs_kernel(int32_t S, const float* __restrict__ dirs_local, flo
     }
 }
 
-// Importance-sampled world directions (x, y, z, pdf) -> (x, y, z, 1/pdf).
-__global__ void world_dirs_kernel(int32_t S, const float4* __restrict__ dirs_world, float4* __restrict__ out4)
+// The probe grid and the tables of one query, by block: [0, n_grid) the grid,
+// then n_dirs blocks of directions, n_env of environment footprints, and the
+// rest of atlas footprints. They are independent of one another, and the
+// first, a serial chain, runs beside the others; seven launches before.
+struct TablesK {
+    const float* probe_pos;
+    int32_t P, g_axis;
+    ProbeGrid* grid;
+    int32_t *cell_start, *cell_cnt;
+    int4* entries;
+    const float* env;
+    int32_t He, We, env_layout;
+    float4* envq;
+    const void* atlas;
+    int32_t R, dtype, what;
+    void* quads;
+    const float* dirs_in;
+    int32_t S, dir_world;
+    float4* dirs;
+    unsigned n_grid, n_dirs, n_env;
+    unsigned int* status;
+};
+
+__global__ void __launch_bounds__(kGridThreads) query_tables_kernel(const TablesK k)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S) return;
-    const float4 d = dirs_world[i];
-    out4[i] = make_float4(d.x, d.y, d.z, 1.f / d.w);
+    __shared__ GridSmem sm;
+    unsigned b = blockIdx.x;
+    if (b < k.n_grid) {
+        probe_grid_build(sm, k.probe_pos, k.P, k.g_axis, k.grid, k.cell_start, k.cell_cnt, k.entries);
+        return;
+    }
+    b -= k.n_grid;
+    if (b < k.n_dirs) {
+        const int i = b * kGridThreads + threadIdx.x;
+        if (i >= k.S) return;
+        if (k.dir_world) {
+            // importance-sampled (x, y, z, pdf) -> (x, y, z, 1/pdf)
+            const float4 d = reinterpret_cast<const float4*>(k.dirs_in)[i];
+            k.dirs[i] = make_float4(d.x, d.y, d.z, 1.f / d.w);
+        } else {
+            const float3 d = local_dir(i, k.S, k.dirs_in);
+            k.dirs[i] = make_float4(d.x, d.y, d.z, 0.f);
+        }
+        return;
+    }
+    b -= k.n_dirs;
+    if (b < k.n_env) {
+        const int64_t i = (int64_t)b * kGridThreads + threadIdx.x;
+        if (!k.envq) {  // checked only
+            if (i < (int64_t)k.He * k.We) {
+                const float3 e = load3(k.env, i);
+                flag_nonfinite(isfinite(e.x + e.y + e.z), k.status);
+            }
+        } else if (k.env_layout == SOP_ENV_OCTAHEDRAL) {
+            if (i < (int64_t)(k.He + 1) * (k.He + 1)) env_oct_footprint(k.env, k.He, i, k.envq, k.status);
+        } else if (i < (int64_t)(k.He + 1) * k.We) {
+            env_footprint(k.env, k.He, k.We, i, k.envq, k.status);
+        }
+        return;
+    }
+    b -= k.n_env;
+    const int64_t i = (int64_t)b * kGridThreads + threadIdx.x;
+    if (i >= (int64_t)k.P * (k.R + 1) * (k.R + 1)) return;
+    if (k.dtype == SOP_F32)
+        atlas_footprint<SOP_F32>(reinterpret_cast<const float4*>(k.atlas), k.R, i, k.what, k.quads, k.status);
+    else if (k.dtype == SOP_BF16)
+        atlas_footprint<SOP_BF16>(reinterpret_cast<const uint2*>(k.atlas), k.R, i, k.what, k.quads, k.status);
+    else atlas_footprint<SOP_F16>(reinterpret_cast<const uint2*>(k.atlas), k.R, i, k.what, k.quads, k.status);
 }
 
 // 256-bit read-only global load (sm_100+); p must be 32-byte aligned.
@@ -1191,75 +1472,90 @@ cudaError_t launch_hammersley(int32_t S, float* out3, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_query_prep(const QueryArgs& a, const QueryLayout& L, char* ws, cudaStream_t s)
+// Up to this many probes a warp a point takes all of them, without a grid.
+constexpr int32_t kKnnAllProbes = 256;
+// Up to this many points a warp a point; above, a thread a point, which
+// issues fewer instructions in all where neighbouring points lie together.
+// Whole calls with one light direction, us (thread / warp): 1,000 points 109 /
+// 69, 8,191: 105 / 77, 32,768: 119 / 126 in pixel order, 128 / 126 at random,
+// 65,536: 136 / 193, 170 / 194.
+constexpr int64_t kKnnWarpPoints = 24576;
+
+static bool knn_needs_grid(int32_t P, int64_t M) { return M > kKnnWarpPoints || P > kKnnAllProbes; }
+
+static cudaError_t launch_knn(const KnnK& k, cudaStream_t s)
 {
-    ProbeGrid* grid = reinterpret_cast<ProbeGrid*>(ws + L.grid_hdr);
-    int32_t* cstart = reinterpret_cast<int32_t*>(ws + L.cell_start);
-    int32_t* ccnt = reinterpret_cast<int32_t*>(ws + L.cell_cnt);
-    int4* ent = reinterpret_cast<int4*>(ws + L.entries);
-    unsigned int* status = status_word();
-    probe_grid_kernel<<<1, 1024, 0, s>>>(a.probe_pos, a.P, L.g_axis, grid, cstart, ccnt, ent);
-    int32_t* idx = reinterpret_cast<int32_t*>(ws + L.idx);
-    float* w = reinterpret_cast<float*>(ws + L.w);
-    if (a.M > 0) {
-        const int bs = 128;
-        const unsigned nb = (unsigned)((a.M + bs - 1) / bs);
-#define SOP_KNN(KM) \
-    knn_kernel<KM><<<nb, bs, 0, s>>>(a.x, a.n, a.M, a.K, a.snap_key, a.r2_key, grid, cstart, ent, a.probe_pos, idx, w, \
-                                     a.out_idx, a.out_w, status)
-        if (a.K <= 4) SOP_KNN(4);
-        else if (a.K <= 8) SOP_KNN(8);
-        else if (a.K <= 16) SOP_KNN(16);
-        else SOP_KNN(32);
+    if (k.M <= kKnnWarpPoints) {
+        knn_warp_kernel<<<(unsigned)((k.M + kKnnWarps - 1) / kKnnWarps), kKnnWarps * 32, 0, s>>>(k);
+        return cudaGetLastError();
+    }
+    const int bs = 128;
+    const unsigned nb = (unsigned)((k.M + bs - 1) / bs);
+#define SOP_KNN(KM)                                                                                                    \
+    knn_kernel<KM><<<nb, bs, 0, s>>>(k.x, k.nrm, k.M, k.K, k.snap_key, k.r2_key, k.grid, k.cell_start, k.entries,      \
+                                     k.probe_pos, k.ws_idx, k.ws_w, k.user_idx, k.user_w, k.status)
+    if (k.K <= 4) SOP_KNN(4);
+    else if (k.K <= 8) SOP_KNN(8);
+    else if (k.K <= 16) SOP_KNN(16);
+    else SOP_KNN(32);
 #undef SOP_KNN
-    }
-    if (a.env_layout == SOP_ENV_OCTAHEDRAL) {
-        const int64_t nq = (int64_t)(a.He + 1) * (a.He + 1);
-        env_oct_quad_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(a.env, a.He,
-                                                                         reinterpret_cast<float4*>(ws + L.envq), status);
-    } else {
-        const int64_t ne = (int64_t)(a.He + 2) * (a.We + 1);
-        env_pack_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(a.env, a.He, a.We,
-                                                                       reinterpret_cast<float4*>(ws + L.env4), status);
-        const int64_t nq = (int64_t)(a.He + 1) * a.We;
-        env_quad_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(reinterpret_cast<const float4*>(ws + L.env4),
-                                                                       a.He, a.We,
-                                                                       reinterpret_cast<float4*>(ws + L.envq));
-    }
-    const int64_t na = (int64_t)a.P * (a.R + 1) * (a.R + 1);
-    const unsigned nba = (unsigned)((na + 255) / 256);
-    if (a.mode == SOP_MODE_SHADOW) {
-        // occlusion-only footprints (a quarter of the RGBO ones, same slot)
-        if (a.rgbo_dtype == SOP_F32)
-            atlas_occ_quad_f32_kernel<<<nba, 256, 0, s>>>(reinterpret_cast<const float4*>(a.rgbo), a.P, a.R,
-                                                          reinterpret_cast<float4*>(ws + L.quads), status);
-        else if (a.rgbo_dtype == SOP_BF16)
-            atlas_occ_quad_16_kernel<SOP_BF16><<<nba, 256, 0, s>>>(reinterpret_cast<const uint2*>(a.rgbo), a.P, a.R,
-                                                                   reinterpret_cast<uint2*>(ws + L.quads), status);
-        else
-            atlas_occ_quad_16_kernel<SOP_F16><<<nba, 256, 0, s>>>(reinterpret_cast<const uint2*>(a.rgbo), a.P, a.R,
-                                                                  reinterpret_cast<uint2*>(ws + L.quads), status);
-    } else switch (a.rgbo_dtype) {
-    case SOP_F32:
-        atlas_quad_kernel<SOP_F32><<<nba, 256, 0, s>>>(reinterpret_cast<const float4*>(a.rgbo), a.P, a.R,
-                                                      reinterpret_cast<float4*>(ws + L.quads), status);
-        break;
-    case SOP_BF16:
-        atlas_quad_kernel<SOP_BF16><<<nba, 256, 0, s>>>(reinterpret_cast<const uint2*>(a.rgbo), a.P, a.R,
-                                                       reinterpret_cast<uint2*>(ws + L.quads), status);
-        break;
-    default:
-        atlas_quad_kernel<SOP_F16><<<nba, 256, 0, s>>>(reinterpret_cast<const uint2*>(a.rgbo), a.P, a.R,
-                                                      reinterpret_cast<uint2*>(ws + L.quads), status);
-        break;
-    }
-    if (a.dir_world)
-        world_dirs_kernel<<<(a.S + 127) / 128, 128, 0, s>>>(a.S, reinterpret_cast<const float4*>(a.dirs_local),
-                                                            reinterpret_cast<float4*>(ws + L.dirs));
-    else
-        dirs_kernel<<<(a.S + 127) / 128, 128, 0, s>>>(a.S, a.dirs_local, reinterpret_cast<float4*>(ws + L.dirs),
-                                                      nullptr);
     return cudaGetLastError();
+}
+
+static bool shade_by_point(const QueryArgs& a);
+
+cudaError_t launch_query_prep(const QueryArgs& a, const QueryLayout& L, char* ws, bool backward, cudaStream_t s)
+{
+    const auto blocks = [](int64_t n) { return (unsigned)((n + kGridThreads - 1) / kGridThreads); };
+    const bool grid = a.M > 0 && knn_needs_grid(a.P, a.M);
+    TablesK t;
+    t.probe_pos = a.probe_pos;
+    t.P = a.P;
+    t.g_axis = L.g_axis;
+    t.grid = reinterpret_cast<ProbeGrid*>(ws + L.grid_hdr);
+    t.cell_start = reinterpret_cast<int32_t*>(ws + L.cell_start);
+    t.cell_cnt = reinterpret_cast<int32_t*>(ws + L.cell_cnt);
+    t.entries = reinterpret_cast<int4*>(ws + L.entries);
+    t.env = a.env;
+    t.He = a.He;
+    t.We = a.We;
+    t.env_layout = a.env_layout;
+    t.envq = backward ? nullptr : reinterpret_cast<float4*>(ws + L.envq);  // the adjoint reads the environment itself
+    t.atlas = a.rgbo;
+    t.R = a.R;
+    t.dtype = a.rgbo_dtype;
+    t.what = backward || shade_by_point(a) ? kAtlasCheck : (a.mode == SOP_MODE_SHADOW ? kAtlasOcc : kAtlasQuads);
+    t.quads = ws + L.quads;
+    t.dirs_in = a.dirs_local;
+    t.S = a.S;
+    t.dir_world = a.dir_world;
+    t.dirs = reinterpret_cast<float4*>(ws + L.dirs);
+    t.status = status_word();
+    t.n_grid = grid ? 1u : 0u;
+    t.n_dirs = blocks(a.S);
+    t.n_env = blocks(!t.envq ? (int64_t)a.He * a.We
+                             : (int64_t)(a.He + 1) * (a.env_layout == SOP_ENV_OCTAHEDRAL ? a.He + 1 : a.We));
+    const int64_t n_atlas = (int64_t)a.P * (a.R + 1) * (a.R + 1);
+    query_tables_kernel<<<t.n_grid + t.n_dirs + t.n_env + blocks(n_atlas), kGridThreads, 0, s>>>(t);
+    if (a.M == 0) return cudaGetLastError();
+    KnnK k;
+    k.x = a.x;
+    k.nrm = a.n;
+    k.M = a.M;
+    k.K = a.K;
+    k.P = a.P;
+    k.snap_key = a.snap_key;
+    k.r2_key = a.r2_key;
+    k.grid = t.grid;
+    k.cell_start = t.cell_start;
+    k.entries = grid ? t.entries : nullptr;
+    k.probe_pos = a.probe_pos;
+    k.ws_idx = reinterpret_cast<int32_t*>(ws + L.idx);
+    k.ws_w = reinterpret_cast<float*>(ws + L.w);
+    k.user_idx = a.out_idx;
+    k.user_w = a.out_w;
+    k.status = t.status;
+    return launch_knn(k, s);
 }
 
 template <int DT, int KMAX, int MODE>
@@ -1462,6 +1758,7 @@ __global__ void sites_setup_kernel(int32_t* mm, int64_t cap, ProbeGrid* grid)
             nc *= G.dims[a];
         }
         G.ncells = nc;
+        G.inv = 0xffffffffu / (uint32_t)G.cs;
         *grid = G;
     }
 }
@@ -1876,17 +2173,24 @@ cudaError_t launch_query_noalloc(const QueryArgs& a, cudaStream_t s)
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int64_t m0 = 0; m0 < a.M; m0 += kNoAllocChunk) {
         const int64_t mc = a.M - m0 < kNoAllocChunk ? a.M - m0 : kNoAllocChunk;
-        const unsigned nb = (unsigned)((mc + 127) / 128);
-        int32_t* uidx = a.out_idx ? a.out_idx + m0 * a.K : nullptr;
-        float* uw = a.out_w ? a.out_w + m0 * a.K : nullptr;
-#define SOP_KNN_NA(KM)                                                                                             \
-    knn_kernel<KM><<<nb, 128, 0, s>>>(a.x + 3 * m0, a.n + 3 * m0, mc, a.K, a.snap_key, a.r2_key, grid, cstart, ent, \
-                                      a.probe_pos, idx, w, uidx, uw, status_word())
-        if (a.K <= 4) SOP_KNN_NA(4);
-        else if (a.K <= 8) SOP_KNN_NA(8);
-        else if (a.K <= 16) SOP_KNN_NA(16);
-        else SOP_KNN_NA(32);
-#undef SOP_KNN_NA
+        KnnK kn;
+        kn.x = a.x + 3 * m0;
+        kn.nrm = a.n + 3 * m0;
+        kn.M = mc;
+        kn.K = a.K;
+        kn.P = a.P;
+        kn.snap_key = a.snap_key;
+        kn.r2_key = a.r2_key;
+        kn.grid = grid;
+        kn.cell_start = cstart;
+        kn.entries = ent;
+        kn.probe_pos = a.probe_pos;
+        kn.ws_idx = idx;
+        kn.ws_w = w;
+        kn.user_idx = a.out_idx ? a.out_idx + m0 * a.K : nullptr;
+        kn.user_w = a.out_w ? a.out_w + m0 * a.K : nullptr;
+        kn.status = status_word();
+        if ((e = launch_knn(kn, s)) != cudaSuccess) return e;
         ShadeDirectK k;
         k.n = a.n + 3 * m0;
         k.wo = a.wo + 3 * m0;

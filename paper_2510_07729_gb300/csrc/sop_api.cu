@@ -389,7 +389,7 @@ sop_status sop_query_shade(const float* x, const float* n, const float* wo, cons
     a.out_idx = out_idx;
     a.out_w = out_w;
     cudaStream_t s = (cudaStream_t)stream;
-    st = cuda_status(sop::launch_query_prep(a, L, (char*)ws, s), "sop_query_shade (prep)");
+    st = cuda_status(sop::launch_query_prep(a, L, (char*)ws, false, s), "sop_query_shade (prep)");
     if (st != SOP_OK) return st;
     return cuda_status(sop::launch_shade(a, L, (char*)ws, s), "sop_query_shade (shade)");
 }
@@ -423,7 +423,7 @@ sop_status sop_query_shade_backward(const float* x, const float* n, const float*
     a.g_env = g_env;
     a.g_atlas = g_maps;
     cudaStream_t s = (cudaStream_t)stream;
-    st = cuda_status(sop::launch_query_prep(a, L, (char*)ws, s), "sop_query_shade_backward (prep)");
+    st = cuda_status(sop::launch_query_prep(a, L, (char*)ws, true, s), "sop_query_shade_backward (prep)");
     if (st != SOP_OK) return st;
     return cuda_status(sop::launch_adjoint(a, L, (char*)ws, s), "sop_query_shade_backward");
 }

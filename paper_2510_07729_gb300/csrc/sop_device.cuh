@@ -155,7 +155,21 @@ struct ProbeGrid {
     int32_t cs;      // cell edge in quantised units (2^-20)
     int32_t dims[3];
     int32_t ncells;
+    uint32_t inv;    // floor((2^32 - 1) / cs)
 };
+
+// x / d with inv = floor((2^32 - 1) / d): the product's high word is at most
+// two below the quotient.
+__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t d, uint32_t inv)
+{
+    uint32_t q = __umulhi(x, inv), r = x - q * d;
+    if (r >= d) {
+        ++q;
+        r -= d;
+    }
+    if (r >= d) ++q;
+    return q;
+}
 
 // Uniform grid over Gaussian bounding spheres, for the bake.
 struct GaussGrid {

@@ -15,7 +15,7 @@ struct GaussGrid;
 
 // ---- query ----------------------------------------------------------------
 struct QueryLayout {
-    size_t grid_hdr, cell_start, cell_cnt, entries, env4, envq, quads, dirs, idx, w, perm, bucket, genv4, total;
+    size_t grid_hdr, cell_start, cell_cnt, entries, envq, quads, dirs, idx, w, perm, bucket, genv4, total;
     int32_t cells_cap, g_axis;
 };
 QueryLayout query_layout(int32_t P, int64_t M, int32_t K, int32_t S, int32_t He, int32_t We, int32_t R,
@@ -44,8 +44,8 @@ struct QueryArgs {
 };
 
 // Enqueue the probe grid, nearest-probe search + weights, environment and
-// direction tables (shared by forward and backward).
-cudaError_t launch_query_prep(const QueryArgs& a, const QueryLayout& L, char* ws, cudaStream_t s);
+// direction tables (the adjoint needs no footprint tables, only the checks).
+cudaError_t launch_query_prep(const QueryArgs& a, const QueryLayout& L, char* ws, bool backward, cudaStream_t s);
 cudaError_t launch_shade(const QueryArgs& a, const QueryLayout& L, char* ws, cudaStream_t s);
 cudaError_t launch_adjoint(const QueryArgs& a, const QueryLayout& L, char* ws, cudaStream_t s);
 cudaError_t launch_hammersley(int32_t S, float* out3, cudaStream_t s);

@@ -117,3 +117,40 @@ def test_shade_and_adjoint_shapes(sop, orc, M, P, R, K, S, caller_dirs):
     for got, ref in ((g["env"], w["env"]), (g["maps"][..., :3], w["maps_rgb"]), (g["maps"][..., 3], w["maps_occ"])):
         d = np.abs(got.cpu().numpy() - ref)
         assert np.all(d <= 1e-4 * np.abs(ref) + 2e-5 * np.abs(ref).max() + 1e-12)
+
+
+@pytest.mark.parametrize("M,P,K,radius", [
+    (1, 1, 1, 0.0), (33, 3, 3, 0.0), (100, 256, 8, 0.0), (100, 257, 8, 0.0), (2000, 4096, 32, 0.0), (500, 1000, 8, 0.05),
+    (24_576, 300, 5, 0.0), (24_577, 300, 5, 0.0), (24_577, 20, 16, 0.3), (3000, 9000, 8, 0.0), (40_000, 30_000, 8, 0.0),
+])
+@pytest.mark.parametrize("layout", ["volume", "sheet", "point"])
+def test_nearest_probes_exact(sop, orc, M, P, K, radius, layout):
+    """Probe indices bit-exact on both sides of every rule: all probes
+    without a grid (up to 256), a warp or a thread a point (24,576 points),
+    grids in shared memory or in the workspace (8,192 cells), flat and
+    degenerate probe sets, ties (every tenth probe twice), points outside."""
+    rng = np.random.default_rng(P + K)
+    pp = rng.uniform(-1, 1, (P, 3))
+    if layout == "sheet":
+        pp[:, 2] = 0.25
+    elif layout == "point":
+        pp[:] = pp[:1] + 1e-6 * rng.integers(0, 2, (P, 3))
+    pp[9::10] = pp[8::10][:len(pp[9::10])]
+    pp = pp.astype(F)
+    x = rng.uniform(-1.5, 1.5, (M, 3)).astype(F)
+    x[::7] = pp[rng.integers(0, P, len(x[::7]))]  # on a probe
+    n = rng.standard_normal((M, 3))
+    n = (n / np.linalg.norm(n, axis=1, keepdims=True)).astype(F)
+    z1, z3 = np.full(M, 0.5, F), np.full((M, 3), 0.5, F)
+    at = sop.make_atlas(cuda(pp), 2, with_depth=False)
+    sop.atlas_pack(cuda(np.zeros((P, 2, 2, 3), F)), cuda(np.zeros((P, 2, 2), F)), None, at)
+    env = np.ones((2, 4, 3), F)
+    _, idx, w = sop.query_shade(cuda(x), cuda(n), cuda(n), cuda(z3), cuda(z1), cuda(z1), at, cuda(env), K, 1,
+                                mode=sop.MODE_SHADOW, return_idx=True, radius=radius)
+    _, oi, ow = orc.query_shade(x, n, n, z3, z1, z1, pp, np.zeros((P, 2, 2, 3), F), np.zeros((P, 2, 2), F), env, K, 1,
+                                mode=orc.MODE_SHADOW, radius=radius)
+    assert np.array_equal(idx.cpu().numpy(), oi)
+    near = np.abs(w.cpu().numpy() - ow) <= 1e-5 * np.abs(ow).max(initial=1e-3)
+    # (probes within a few ulp of a point: 1/d itself is not resolved in float32)
+    d = np.linalg.norm(pp[np.clip(oi[:, 0], 0, None)].astype(np.float64) - x, axis=1)
+    assert near[d > 1e-3].all()
