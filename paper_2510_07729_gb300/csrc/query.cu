@@ -12,7 +12,9 @@
 //                        directions, 4 texel fetches per probe and direction
 //                        from the L2-resident footprints), shade_point_kernel
 //                        (a warp a point, probes blended first),
-//                        shade_world_kernel (importance-sampled directions).
+//                        shadow_warp_kernel (SHADOW: points on one normal
+//                        share each probe's integral), shade_world_kernel
+//                        (importance-sampled directions).
 #include <float.h>
 #include <stdlib.h>
 
@@ -1178,6 +1180,208 @@ __global__ void __launch_bounds__(256, 4) shade_kernel(const ShadeK a, const int
 }
 
 // ---------------------------------------------------------------------------
+// SHADOW mode, large calls: one thread per point.
+//
+// The shadow ratio is 1 - sum_i L_i cos_i O(w_i) / sum_i L_i cos_i with O =
+// sum_k W_k O_k (Eq. 5 applied to O), so the sum over directions can be taken
+// per probe first: V_k = sum_i L_i cos_i O_k(w_i), ratio = 1 - sum_k W_k V_k /
+// den. V_k depends on the point only through its normal. Where the points of
+// a warp share one normal bit for bit (a planar receiver such as a ground
+// plane: their directions, footprints and environment terms coincide), the
+// warp takes each of its distinct probes once, the lanes over the directions,
+// and the 32 points combine the results: a few probes times S footprints a
+// warp instead of 32 K S. Neighbouring points share nearly all their probes
+// (about 10 distinct of 256); a warp with more than kShadowProbes of them, or
+// with several normals, blends per point and direction as shade_kernel does.
+// Bound: the reads of normals, indices and weights, then issue. 2,051,693
+// ground points, K = 8, S = 64, 16-bit atlas: 716 -> 255 us.
+// ---------------------------------------------------------------------------
+constexpr int kShadowProbes = 32;
+// Whole calls, us (lanes / warp): 16-bit atlas, S 64: 32,768 points 163 / 208,
+// 131,072: 208 / 217 (on a ground), 248 / 260 (on an object: mixed normals),
+// float32 on an object 284 / 274; 2,051,693 on a ground: 1,240 / 776. A warp's
+// few serial steps do not fill the machine below.
+constexpr int64_t kShadowWarpPoints = 262144;
+
+// Ratio of one point by blending per direction, LANES threads a point.
+template <int DT, int KMAX, int LANES>
+__device__ __forceinline__ void shadow_point(const ShadeK& a, const float4* __restrict__ s_dirs, const int64_t m,
+                                             const int sub, const bool active)
+{
+    const int64_t mm = active ? m : 0;
+    const float3 nr = load3(a.n, mm);
+    const float nl = sqrtf(dot3(nr, nr));
+    const float3 n = f3(nr.x / nl, nr.y / nl, nr.z / nl);
+    float3 tt, bb;
+    onb(n, tt, bb);
+    const int RQ = a.R + 1;
+    int32_t base[KMAX];
+    float W[KMAX];
+#pragma unroll
+    for (int k = 0; k < KMAX; ++k) {
+        const bool on = k < a.K;
+        base[k] = on ? __ldg(a.idx + mm * a.K + k) * RQ * RQ : 0;
+        W[k] = on ? __ldg(a.w + mm * a.K + k) : 0.f;
+    }
+    float acc[3] = {0.f, 0.f, 0.f}, den[3] = {0.f, 0.f, 0.f};
+    const float Rf = (float)a.R;
+    for (int i = sub; i < a.S; i += LANES) {
+        const float4 l = s_dirs[i];
+        const DirTerms d = dir_terms(l, tt, bb, n, Rf, a.R, RQ);
+        const float vis = 1.f - shadow_blend<DT, KMAX>(a.quads, base, W, a.K, d.off, d.w00, d.w10, d.w01, d.w11);
+        const float3 Ld = a.env_layout == SOP_ENV_OCTAHEDRAL ? env_oct_lookup(a.envq, a.He, d.uv)
+                                                             : env_lookup(a.envq, a.He, a.We, d.w);
+        const float L[3] = {Ld.x * l.z, Ld.y * l.z, Ld.z * l.z};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            acc[c] = fmaf(L[c], vis, acc[c]);
+            den[c] += L[c];
+        }
+    }
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+            den[c] += __shfl_xor_sync(0xffffffffu, den[c], o);
+        }
+    if (active && sub == 0)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a.out[3 * m + c] = den[c] < 1e-20f ? 1.f : acc[c] / den[c];
+}
+
+template <int DT, int KMAX>
+__global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
+{
+    extern __shared__ float4 s_dirs[];
+    for (int i = threadIdx.x; i < a.S; i += blockDim.x) s_dirs[i] = a.dirs[i];
+    __syncthreads();
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int64_t m0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~(int64_t)31;  // the warp's first point
+    if (m0 >= a.M) return;
+    const int64_t m = m0 + lane;
+    const bool active = m < a.M;
+    const int64_t mm = active ? m : a.M - 1;
+    const float3 nr = load3(a.n, mm);
+    // every lane takes all three shuffles (no short-circuit)
+    const unsigned bx = __float_as_uint(nr.x), by = __float_as_uint(nr.y), bz = __float_as_uint(nr.z);
+    const unsigned x0 = __shfl_sync(full, bx, 0), y0 = __shfl_sync(full, by, 0), z0 = __shfl_sync(full, bz, 0);
+    bool shared = __all_sync(full, (bx == x0) & (by == y0) & (bz == z0));
+    const int RQ = a.R + 1;
+    int32_t id[KMAX];
+    float W[KMAX];
+    if (shared) {
+        // the warp's distinct probes, ascending, one a lane
+        int32_t mine = 0, last = -1;
+        int n = 0;
+#pragma unroll
+        for (int k = 0; k < KMAX; ++k) {
+            const bool on = k < a.K;
+            id[k] = on ? __ldg(a.idx + mm * a.K + k) : INT32_MAX;
+            W[k] = on ? __ldg(a.w + mm * a.K + k) : 0.f;
+        }
+        for (;; ++n) {
+            int32_t next = INT32_MAX;
+#pragma unroll
+            for (int k = 0; k < KMAX; ++k) next = min(next, id[k] > last ? id[k] : INT32_MAX);
+            next = __reduce_min_sync(full, next);
+            if (next == INT32_MAX || n == kShadowProbes) {
+                shared = next == INT32_MAX;
+                break;
+            }
+            if (lane == n) mine = next;
+            last = next;
+        }
+        if (shared) {
+            const float nl = sqrtf(dot3(nr, nr));
+            const float3 nn = f3(nr.x / nl, nr.y / nl, nr.z / nl);
+            float3 tt, bb;
+            onb(nn, tt, bb);
+            // this lane's directions: footprint, weights, environment times cos
+            constexpr int NR = kShadowTab / 32;
+            int off[NR];
+            float fu[NR], fv[NR], L[NR][3], den[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int i = r * 32 + lane;
+                off[r] = -1;
+                if (i < a.S) {
+                    const float4 l = s_dirs[i];
+                    const DirTerms d = dir_terms(l, tt, bb, nn, (float)a.R, a.R, RQ);
+                    const float3 Ld = a.env_layout == SOP_ENV_OCTAHEDRAL ? env_oct_lookup(a.envq, a.He, d.uv)
+                                                                         : env_lookup(a.envq, a.He, a.We, d.w);
+                    off[r] = d.off;
+                    fu[r] = d.w10 + d.w11;
+                    fv[r] = d.w01 + d.w11;
+                    L[r][0] = Ld.x * l.z;
+                    L[r][1] = Ld.y * l.z;
+                    L[r][2] = Ld.z * l.z;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) den[c] += L[r][c];
+                }
+            }
+            // two probes a step: their loads overlap, and the sums over the
+            // lanes go on in one half of the warp each
+            float num[3] = {0.f, 0.f, 0.f};
+            const bool lower = lane < 16;
+            for (int u = 0; u < n; u += 2) {
+                int32_t p[2];
+                float V[2][3], w[2] = {0.f, 0.f};
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    p[j] = __shfl_sync(full, mine, min(u + j, n - 1));
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) V[j][c] = 0.f;
+                }
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (off[r] >= 0) {
+                        const float4 qa = OQuad<DT>::load(a.quads, (int64_t)(p[0] * RQ * RQ + off[r]));
+                        const float4 qb = OQuad<DT>::load(a.quads, (int64_t)(p[1] * RQ * RQ + off[r]));
+                        const float la = fmaf(fu[r], qa.y - qa.x, qa.x), ha = fmaf(fu[r], qa.w - qa.z, qa.z);
+                        const float lb = fmaf(fu[r], qb.y - qb.x, qb.x), hb = fmaf(fu[r], qb.w - qb.z, qb.z);
+                        const float Oa = fmaf(fv[r], ha - la, la), Ob = fmaf(fv[r], hb - lb, lb);
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            V[0][c] = fmaf(L[r][c], Oa, V[0][c]);
+                            V[1][c] = fmaf(L[r][c], Ob, V[1][c]);
+                        }
+                    }
+#pragma unroll
+                for (int k = 0; k < KMAX; ++k) {
+                    w[0] += id[k] == p[0] ? W[k] : 0.f;
+                    w[1] += id[k] == p[1] ? W[k] : 0.f;
+                }
+                if (u + 1 == n) w[1] = 0.f;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    float v = (lower ? V[0][c] : V[1][c]) + __shfl_xor_sync(full, lower ? V[1][c] : V[0][c], 16);
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
+                    const float x = __shfl_xor_sync(full, v, 16);
+                    if (w[0] != 0.f) num[c] = fmaf(w[0], lower ? v : x, num[c]);
+                    if (w[1] != 0.f) num[c] = fmaf(w[1], lower ? x : v, num[c]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) den[c] += __shfl_xor_sync(full, den[c], o);
+                if (active) a.out[3 * m + c] = den[c] < 1e-20f ? 1.f : (den[c] - num[c]) / den[c];
+            }
+            return;
+        }
+    }
+    // as many lanes a point as shade_kernel takes
+    constexpr int LANES = DT == SOP_F32 ? 1 : 2;
+    for (int j = 0; j < LANES; ++j) {
+        const int64_t mj = m0 + j * (32 / LANES) + lane / LANES;
+        shadow_point<DT, KMAX, LANES>(a, s_dirs, mj, lane % LANES, mj < a.M);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Query + shade, SHADE mode, one warp per point (point_blend.cuh): lanes
 // share the directions, 32 a round. NR: rounds whose footprints stay in
 // registers between the marking and the shading (S <= 32 NR), or 0: any S,
@@ -1635,9 +1839,22 @@ static bool shade_by_point(const QueryArgs& a)
     return sk >= (a.rgbo_dtype == SOP_F32 ? 3 : 4) * t || (a.M <= kPointSmall && sk >= t);
 }
 
+template <int DT, int KMAX>
+static cudaError_t shadow_warp_launch(const ShadeK& k, cudaStream_t s)
+{
+    shadow_warp_kernel<DT, KMAX><<<(unsigned)((k.M + 255) / 256), 256, sizeof(float4) * (size_t)k.S, s>>>(k);
+    return cudaGetLastError();
+}
+
 template <int DT, int MODE>
 static cudaError_t shade_k(const ShadeK& k, cudaStream_t s)
 {
+    if (MODE == SOP_MODE_SHADOW && k.S <= kShadowTab && k.M >= kShadowWarpPoints) {
+        if (k.K <= 4) return shadow_warp_launch<DT, 4>(k, s);
+        if (k.K <= 8) return shadow_warp_launch<DT, 8>(k, s);
+        if (k.K <= 16) return shadow_warp_launch<DT, 16>(k, s);
+        return shadow_warp_launch<DT, 32>(k, s);
+    }
     if (k.K <= 4) return shade_dispatch<DT, 4, MODE>(k, s);
     if (k.K <= 8) return shade_dispatch<DT, 8, MODE>(k, s);
     if (k.K <= 16) return shade_dispatch<DT, 16, MODE>(k, s);

@@ -154,3 +154,36 @@ def test_nearest_probes_exact(sop, orc, M, P, K, radius, layout):
     # (probes within a few ulp of a point: 1/d itself is not resolved in float32)
     d = np.linalg.norm(pp[np.clip(oi[:, 0], 0, None)].astype(np.float64) - x, axis=1)
     assert near[d > 1e-3].all()
+
+
+@pytest.mark.parametrize("M", [262_143, 262_144, 262_175])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+@pytest.mark.parametrize("K,S", [(8, 64), (4, 33), (12, 128)])
+def test_shadow_shared_integrals(sop, orc, M, dtype, K, S):
+    """SHADOW on both sides of the size from which warps on one normal share
+    their probes' integrals; warps with one normal, with two, and with more
+    distinct probes than a warp keeps. A sample against the oracle: 1e-5 plus
+    the sensitivity, on maps that are exact in 16 bits."""
+    P, R = 600, 8
+    rng = np.random.default_rng(S)
+    pp = np.concatenate([rng.uniform(-1, 1, (P, 2)), np.full((P, 1), 0.02)], axis=1).astype(F)
+    x = np.zeros((M, 3), F)
+    x[:, 0] = np.linspace(-1.1, 1.1, M)
+    x[:, 1] = 0.3 * np.sin(5 * x[:, 0])
+    x[M // 2: M // 2 + 4096] = rng.uniform(-1, 1, (4096, 3)) * [1, 1, 0]  # scattered: many probes a warp
+    n = np.tile(np.array([0.0, 0.0, 1.0], F), (M, 1))
+    n[5000:5040:3] = np.array([0.6, 0.0, 0.8], F)  # mixed normals in two warps
+    occ = (rng.integers(0, 65, (P, R, R)) / 64).astype(F)
+    rgb = np.zeros((P, R, R, 3), F)
+    env = np.exp(0.3 * np.sin(np.arange(16 * 32 * 3).reshape(16, 32, 3) / 50.0)).astype(F)
+    one = np.full(M, 0.5, F)
+    at = sop.make_atlas(cuda(pp), R, dtype, with_depth=False)
+    sop.atlas_pack(cuda(rgb), cuda(occ), None, at)
+    dev = [cuda(v) for v in (x, n, n, np.full((M, 3), 0.5, F), one, one)]
+    out = sop.query_shade(*dev, at, cuda(env), K, S, mode=sop.MODE_SHADOW).cpu().numpy()
+    sel = np.unique(np.concatenate([rng.integers(0, M, 300), np.arange(4990, 5045), np.arange(M // 2, M // 2 + 200),
+                                    np.arange(M - 70, M)]))
+    args = [x[sel], n[sel], n[sel], np.full((len(sel), 3), 0.5, F), one[sel], one[sel], pp, rgb, occ, env, K, S]
+    want, _, _ = orc.query_shade(*args, mode=orc.MODE_SHADOW)
+    sens = orc.query_shade_sensitivity(*args, mode=orc.MODE_SHADOW)
+    assert np.all(np.abs(out[sel] - want) <= 1e-5 * np.maximum(np.abs(want), 1e-3 * np.abs(want).mean()) + sens)
