@@ -1007,7 +1007,7 @@ def main():
         "query": {"ms": round(mq, 4), "point_dirs_per_s": round(pd / (mq * 1e-3), 1) if do_query else None,
                   "parts": {q["name"]: q["M"] for q in st.parts}},
         "wall_s_timed_region": round(r["wall_s"], 4),
-        "gpu_launches": launches_per_step(do_bake, len(st.parts) if do_query else 0) * args.steps,
+        "gpu_launches": step_launches(do_bake, len(st.parts) if do_query else 0) * args.steps,
         "clocks": r["clocks"],
         "roofline": roof,
         "roofline_query": frame["fp32"]["roofline"] if frame else None,
@@ -1083,17 +1083,22 @@ def compose_only(args, dev, sop):
 
 
 def launches_per_step(do_bake, n_queries):
-    """This library's kernel launches in one step."""
+    """Kernel launches of the step in the recorded launch list
+    (profiles/launches_compose_step.md), taken when binning, tables and
+    search were 29 launches; step_launches() counts the present ones."""
+    return (22 if do_bake else 0) + 7 * n_queries
+
+
+def step_launches(do_bake, n_queries):
+    """This library's kernel launches in one step (more than 4,096 Gaussians)."""
     n = 0
     if do_bake:
-        # binning: bbox init, Gaussian records, 3 attempts x (grid setup,
-        # count, and the scan's tile sums, tile offsets and apply) decided on
-        # the device, fill; trace: counter reset, texel directions, trace,
-        # atlas border
-        n += 2 + 3 * 5 + 1 + 4
-    # per query: probe grid, nearest probes, environment table and
-    # footprints, atlas footprints, directions, shade
-    n += 7 * n_queries
+        # binning: Gaussian records, grid set-up, count, the scan's tile sums
+        # and apply, the coarser attempts (decided on the device), fill;
+        # trace: counters and texel directions, trace, atlas border
+        n += 7 + 3
+    # per query: probe grid with all tables, nearest probes, shade
+    n += 3 * n_queries
     return n
 
 

@@ -81,144 +81,180 @@ __device__ __forceinline__ int32_t f2o(float f)
 }
 __device__ __forceinline__ float o2f(int32_t i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-__global__ void bbox_init_kernel(int32_t* bbox)
+// Per-Gaussian record; lo and hi take in the box of its alpha_min ellipsoid
+// (margin-expanded). A Gaussian with a non-finite parameter, a scale <= 0 or a
+// zero quaternion is left out of the bake (rho < 0) and flagged in the device
+// status word.
+__device__ __forceinline__ void gauss_record(const sop_gaussians& g, int64_t i, float alpha_min, GRec* __restrict__ rec,
+                                             unsigned int* status, float lo[3], float hi[3])
 {
-    if (threadIdx.x < 3) bbox[threadIdx.x] = f2o(FLT_MAX);
-    else if (threadIdx.x < 6) bbox[threadIdx.x] = f2o(-FLT_MAX);
-    else if (threadIdx.x < 8) bbox[threadIdx.x] = 0;  // [6]: binning status word
+    const float qw = g.quat[4 * i], qx = g.quat[4 * i + 1], qy = g.quat[4 * i + 2], qz = g.quat[4 * i + 3];
+    const float qn = sqrtf(qw * qw + qx * qx + qy * qy + qz * qz);
+    const float w = qw / qn, x = qx / qn, y = qy / qn, z = qz / qn;
+    // rotation matrix (columns = local axes in world space)
+    const float R00 = 1.f - 2.f * (y * y + z * z), R01 = 2.f * (x * y - w * z), R02 = 2.f * (x * z + w * y);
+    const float R10 = 2.f * (x * y + w * z), R11 = 1.f - 2.f * (x * x + z * z), R12 = 2.f * (y * z - w * x);
+    const float R20 = 2.f * (x * z - w * y), R21 = 2.f * (y * z + w * x), R22 = 1.f - 2.f * (x * x + y * y);
+    const float sx = g.scale[3 * i], sy = g.scale[3 * i + 1], sz = g.scale[3 * i + 2];
+    const float ix = 1.f / sx, iy = 1.f / sy, iz = 1.f / sz;
+    const float o = g.opacity[i];
+    const float3 mu = load3(g.mean, i);
+    const float c0 = g.rgb[3 * i], c1 = g.rgb[3 * i + 1], c2 = g.rgb[3 * i + 2];
+    // a NaN anywhere makes the sum NaN; an Inf makes it Inf or NaN
+    const bool ok = isfinite(mu.x + mu.y + mu.z + sx + sy + sz + qw + qx + qy + qz + o + c0 + c1 + c2) &&
+                    sx > 0.f && sy > 0.f && sz > 0.f && qn > 0.f && isfinite(ix + iy + iz);
+    if (!ok && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
+    float rho = -1.f, ex = 0.f, ey = 0.f, ez = 0.f;
+    if (ok && o >= alpha_min && o > 0.f) {
+        // {x : o exp(-m^2(x)/2) >= alpha_min} is the ellipsoid m^2 <= kk^2
+        const float kk = sqrtf(2.f * fmaxf(logf(o / alpha_min), 0.f));
+        const float smax = fmaxf(sx, fmaxf(sy, sz));
+        rho = smax * kk * (1.f + kMarginRel) + 1e-7f;
+        // axis-aligned half extents: kk sqrt(Sigma_aa), Sigma = R diag(s^2) R^T
+        const float sx2 = sx * sx, sy2 = sy * sy, sz2 = sz * sz;
+        ex = kk * sqrtf(R00 * R00 * sx2 + R01 * R01 * sy2 + R02 * R02 * sz2) * (1.f + kMarginRel) + 1e-7f;
+        ey = kk * sqrtf(R10 * R10 * sx2 + R11 * R11 * sy2 + R12 * R12 * sz2) * (1.f + kMarginRel) + 1e-7f;
+        ez = kk * sqrtf(R20 * R20 * sx2 + R21 * R21 * sy2 + R22 * R22 * sz2) * (1.f + kMarginRel) + 1e-7f;
+        ex = fminf(ex, rho);
+        ey = fminf(ey, rho);
+        ez = fminf(ez, rho);
+    }
+    GRec r;
+    r.r0 = make_float4(mu.x, mu.y, mu.z, rho);
+    // M = diag(1/s) R^T : row a = R[:, a] / s_a
+    r.r1 = make_float4(R00 * ix, R10 * ix, R20 * ix, R01 * iy);
+    r.r2 = make_float4(R11 * iy, R21 * iy, R02 * iz, R12 * iz);
+    r.r3 = make_float4(R22 * iz, o, c0, c1);
+    r.r4 = make_float4(c2, ex, ey, ez);
+    rec[i] = r;
+    if (rho >= 0.f) {
+        lo[0] = fminf(lo[0], mu.x - ex);
+        lo[1] = fminf(lo[1], mu.y - ey);
+        lo[2] = fminf(lo[2], mu.z - ez);
+        hi[0] = fmaxf(hi[0], mu.x + ex);
+        hi[1] = fmaxf(hi[1], mu.y + ey);
+        hi[2] = fmaxf(hi[2], mu.z + ez);
+    }
 }
 
-// Per-Gaussian record + bounding box of the (margin-expanded) spheres. A
-// Gaussian with a non-finite parameter, a scale <= 0 or a zero quaternion is
-// left out of the bake (rho < 0) and flagged in the device status word.
-__global__ void gauss_prep_kernel(sop_gaussians g, float alpha_min, GRec* __restrict__ rec, int32_t* bbox,
-                                  unsigned int* status)
+// The box [lo, hi] of a CTA's threads, in every thread of warp 0 (order-
+// preserving ints; smallest 0..2, largest 3..5). s_box: [6][32].
+__device__ __forceinline__ void cta_box(const float lo[3], const float hi[3], int32_t (*s_box)[32], int32_t box[6])
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-    if (i < g.n) {
-        const float qw = g.quat[4 * i], qx = g.quat[4 * i + 1], qy = g.quat[4 * i + 2], qz = g.quat[4 * i + 3];
-        const float qn = sqrtf(qw * qw + qx * qx + qy * qy + qz * qz);
-        const float w = qw / qn, x = qx / qn, y = qy / qn, z = qz / qn;
-        // rotation matrix (columns = local axes in world space)
-        const float R00 = 1.f - 2.f * (y * y + z * z), R01 = 2.f * (x * y - w * z), R02 = 2.f * (x * z + w * y);
-        const float R10 = 2.f * (x * y + w * z), R11 = 1.f - 2.f * (x * x + z * z), R12 = 2.f * (y * z - w * x);
-        const float R20 = 2.f * (x * z - w * y), R21 = 2.f * (y * z + w * x), R22 = 1.f - 2.f * (x * x + y * y);
-        const float sx = g.scale[3 * i], sy = g.scale[3 * i + 1], sz = g.scale[3 * i + 2];
-        const float ix = 1.f / sx, iy = 1.f / sy, iz = 1.f / sz;
-        const float o = g.opacity[i];
-        const float3 mu = load3(g.mean, i);
-        const float c0 = g.rgb[3 * i], c1 = g.rgb[3 * i + 1], c2 = g.rgb[3 * i + 2];
-        // a NaN anywhere makes the sum NaN; an Inf makes it Inf or NaN
-        const bool ok = isfinite(mu.x + mu.y + mu.z + sx + sy + sz + qw + qx + qy + qz + o + c0 + c1 + c2) &&
-                        sx > 0.f && sy > 0.f && sz > 0.f && qn > 0.f && isfinite(ix + iy + iz);
-        if (!ok && status) atomicOr(status, SOP_DEVSTAT_NONFINITE);
-        float rho = -1.f, ex = 0.f, ey = 0.f, ez = 0.f;
-        if (ok && o >= alpha_min && o > 0.f) {
-            // {x : o exp(-m^2(x)/2) >= alpha_min} is the ellipsoid m^2 <= kk^2
-            const float kk = sqrtf(2.f * fmaxf(logf(o / alpha_min), 0.f));
-            const float smax = fmaxf(sx, fmaxf(sy, sz));
-            rho = smax * kk * (1.f + kMarginRel) + 1e-7f;
-            // axis-aligned half extents: kk sqrt(Sigma_aa), Sigma = R diag(s^2) R^T
-            const float sx2 = sx * sx, sy2 = sy * sy, sz2 = sz * sz;
-            ex = kk * sqrtf(R00 * R00 * sx2 + R01 * R01 * sy2 + R02 * R02 * sz2) * (1.f + kMarginRel) + 1e-7f;
-            ey = kk * sqrtf(R10 * R10 * sx2 + R11 * R11 * sy2 + R12 * R12 * sz2) * (1.f + kMarginRel) + 1e-7f;
-            ez = kk * sqrtf(R20 * R20 * sx2 + R21 * R21 * sy2 + R22 * R22 * sz2) * (1.f + kMarginRel) + 1e-7f;
-            ex = fminf(ex, rho);
-            ey = fminf(ey, rho);
-            ez = fminf(ez, rho);
-        }
-        GRec r;
-        r.r0 = make_float4(mu.x, mu.y, mu.z, rho);
-        // M = diag(1/s) R^T : row a = R[:, a] / s_a
-        r.r1 = make_float4(R00 * ix, R10 * ix, R20 * ix, R01 * iy);
-        r.r2 = make_float4(R11 * iy, R21 * iy, R02 * iz, R12 * iz);
-        r.r3 = make_float4(R22 * iz, o, c0, c1);
-        r.r4 = make_float4(c2, ex, ey, ez);
-        rec[i] = r;
-        if (rho >= 0.f) {
-            lo[0] = mu.x - ex; lo[1] = mu.y - ey; lo[2] = mu.z - ez;
-            hi[0] = mu.x + ex; hi[1] = mu.y + ey; hi[2] = mu.z + ez;
-        }
-    }
-    // warp reduce then one atomic per warp
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        for (int off = 16; off > 0; off >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], off));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], off));
+        const int32_t l = __reduce_min_sync(full, f2o(lo[a])), h = __reduce_max_sync(full, f2o(hi[a]));
+        if (lane == 0) {
+            s_box[a][warp] = l;
+            s_box[3 + a][warp] = h;
         }
-    }
-    if ((threadIdx.x & 31) == 0) {
-        for (int a = 0; a < 3; ++a) {
-            if (lo[a] <= hi[a]) {
-                atomicMin(&bbox[a], f2o(lo[a]));
-                atomicMax(&bbox[3 + a], f2o(hi[a]));
-            }
-        }
-    }
-}
-
-// Grid geometry from the bounding box: cubic cells, about cells_cap/2 of
-// them over the box, never more than cells_cap. Binning attempt `level`
-// (> 0: the previous attempt's cell lists did not fit the workspace) does
-// nothing once an earlier attempt fitted.
-__global__ void grid_setup_kernel(const int32_t* bbox, int64_t cells_cap, int32_t level, GaussGrid* grid,
-                                  int32_t* cell_cnt)
-{
-    __shared__ GaussGrid G;
-    if (level > 0 && grid->fits) return;
-    if (threadIdx.x == 0) {
-        float lo[3], hi[3], ext[3];
-        bool empty = false;
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = o2f(bbox[a]);
-            hi[a] = o2f(bbox[3 + a]);
-            if (!(lo[a] <= hi[a])) empty = true;
-        }
-        if (empty) {
-            for (int a = 0; a < 3; ++a) { lo[a] = 0.f; hi[a] = 0.f; }
-        }
-        float emax = 0.f;
-        for (int a = 0; a < 3; ++a) {
-            // pad the box so boundary rounding never drops a sphere
-            const float pad = 1e-5f * fmaxf(hi[a] - lo[a], 1e-3f) + 1e-6f;
-            lo[a] -= pad;
-            hi[a] += pad;
-            ext[a] = hi[a] - lo[a];
-            emax = fmaxf(emax, ext[a]);
-        }
-        // cell edge: volume / (cells_cap/2), clamped so that no axis needs
-        // more than cbrt-balanced resolution
-        const double vol = (double)ext[0] * ext[1] * ext[2];
-        double h = cbrt(vol / (double)(cells_cap / 2));
-        h = fmax(h, (double)emax / 1024.0);
-        int64_t nc;
-        int d[3];
-        for (;;) {
-            nc = 1;
-            for (int a = 0; a < 3; ++a) {
-                d[a] = (int)ceil(ext[a] / h);
-                d[a] = d[a] < 1 ? 1 : d[a];
-                nc *= d[a];
-            }
-            if (nc <= cells_cap) break;
-            h *= 1.1;
-        }
-        for (int a = 0; a < 3; ++a) {
-            G.origin[a] = lo[a];
-            G.bmax[a] = hi[a];
-            G.dims[a] = d[a];
-        }
-        G.h = (float)h;
-        G.inv_h = (float)(1.0 / h);
-        G.ncells = (int32_t)nc;
-        G.n_entries = 0;
-        G.fits = 0;
-        G.level = level;
-        *grid = G;
     }
     __syncthreads();
-    for (int c = threadIdx.x; c < G.ncells; c += blockDim.x) cell_cnt[c] = 0;
+    if (warp == 0)
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+            const int32_t v = lane < warps ? s_box[a][lane] : (a < 3 ? INT32_MAX : INT32_MIN);
+            box[a] = a < 3 ? __reduce_min_sync(full, v) : __reduce_max_sync(full, v);
+        }
+}
+
+// Records, each CTA's box (part[6][parts]: no atomics and nothing to clear
+// first), and the cell counters cleared for the count.
+__global__ void __launch_bounds__(256) gauss_prep_kernel(sop_gaussians g, float alpha_min, GRec* __restrict__ rec,
+                                                         int32_t* __restrict__ part, int32_t* __restrict__ cell_cnt,
+                                                         int64_t cells_cap, unsigned int* status)
+{
+    __shared__ int32_t s_box[6][32];
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t c = i; c < cells_cap; c += (int64_t)gridDim.x * blockDim.x) cell_cnt[c] = 0;
+    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+    if (i < g.n) gauss_record(g, i, alpha_min, rec, status, lo, hi);
+    int32_t box[6];
+    cta_box(lo, hi, s_box, box);
+    if (threadIdx.x < 6) {
+        const int a = threadIdx.x;
+        part[(int64_t)a * gridDim.x + blockIdx.x] =
+            a == 0 ? box[0] : (a == 1 ? box[1] : (a == 2 ? box[2] : (a == 3 ? box[3] : (a == 4 ? box[4] : box[5]))));
+    }
+}
+
+// Grid geometry from the bounding box (order-preserving ints): cubic cells,
+// about cells_cap/2 of them over the box, never more than cells_cap.
+__device__ __forceinline__ GaussGrid grid_geometry(const int32_t box[6], int64_t cells_cap, int32_t level)
+{
+    GaussGrid G;
+    float lo[3], hi[3], ext[3];
+    bool empty = false;
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = o2f(box[a]);
+        hi[a] = o2f(box[3 + a]);
+        if (!(lo[a] <= hi[a])) empty = true;
+    }
+    if (empty) {
+        for (int a = 0; a < 3; ++a) { lo[a] = 0.f; hi[a] = 0.f; }
+    }
+    float emax = 0.f;
+    for (int a = 0; a < 3; ++a) {
+        // pad the box so boundary rounding never drops a sphere
+        const float pad = 1e-5f * fmaxf(hi[a] - lo[a], 1e-3f) + 1e-6f;
+        lo[a] -= pad;
+        hi[a] += pad;
+        ext[a] = hi[a] - lo[a];
+        emax = fmaxf(emax, ext[a]);
+    }
+    // cell edge: volume / (cells_cap/2), clamped so that no axis needs
+    // more than cbrt-balanced resolution
+    const double vol = (double)ext[0] * ext[1] * ext[2];
+    double h = cbrt(vol / (double)(cells_cap / 2));
+    h = fmax(h, (double)emax / 1024.0);
+    int64_t nc;
+    int d[3];
+    for (;;) {
+        nc = 1;
+        for (int a = 0; a < 3; ++a) {
+            d[a] = (int)ceil(ext[a] / h);
+            d[a] = d[a] < 1 ? 1 : d[a];
+            nc *= d[a];
+        }
+        if (nc <= cells_cap) break;
+        h *= 1.1;
+    }
+    for (int a = 0; a < 3; ++a) {
+        G.origin[a] = lo[a];
+        G.bmax[a] = hi[a];
+        G.dims[a] = d[a];
+    }
+    G.h = (float)h;
+    G.inv_h = (float)(1.0 / h);
+    G.ncells = (int32_t)nc;
+    G.n_entries = 0;
+    G.fits = 0;
+    G.level = level;
+    G.pad = 0;
+    return G;
+}
+
+// One CTA: the box of all Gaussians from the CTAs' parts (kept in bbox for a
+// coarser attempt), and the requested grid.
+__global__ void __launch_bounds__(1024) grid_setup_kernel(const int32_t* __restrict__ part, int32_t parts,
+                                                          int64_t cells_cap, int32_t* bbox, GaussGrid* grid)
+{
+    __shared__ int32_t s_box[6][32];
+    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+    for (int i = threadIdx.x; i < parts; i += blockDim.x)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = fminf(lo[a], o2f(part[(int64_t)a * parts + i]));
+            hi[a] = fmaxf(hi[a], o2f(part[(int64_t)(3 + a) * parts + i]));
+        }
+    int32_t box[6];
+    cta_box(lo, hi, s_box, box);
+    if (threadIdx.x == 0) {
+        for (int a = 0; a < 6; ++a) bbox[a] = box[a];
+        *grid = grid_geometry(box, cells_cap, 0);
+    }
 }
 
 // A cell entry is the Gaussian's box as the walk tests it, in 16 bytes: the
@@ -271,14 +307,13 @@ __device__ __forceinline__ void cell_range(const GaussGrid& G, const uint4 en, i
     }
 }
 
-__global__ void bin_count_kernel(int64_t N, const GRec* __restrict__ rec, const GaussGrid* __restrict__ gridp,
-                                 int32_t* __restrict__ cell_cnt)
+// Gaussian i counted in its cells, or entered into them (after the scan of the
+// counts, which clears them).
+__device__ __forceinline__ void bin_count(int64_t i, const GRec* __restrict__ rec, const GaussGrid& G,
+                                          int32_t* __restrict__ cell_cnt)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N || gridp->fits) return;
     const float4 r0 = rec[i].r0;
     if (r0.w < 0.f) return;
-    const GaussGrid G = *gridp;
     int lo[3], hi[3];
     cell_range(G, make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i), lo, hi);
     for (int z = lo[2]; z <= hi[2]; ++z)
@@ -286,11 +321,33 @@ __global__ void bin_count_kernel(int64_t N, const GRec* __restrict__ rec, const 
             for (int x = lo[0]; x <= hi[0]; ++x) atomicAdd(&cell_cnt[(z * G.dims[1] + y) * G.dims[0] + x], 1);
 }
 
-// Exclusive scan of the cell counts in one CTA; total into grid->n_entries,
-// and grid->fits = 1 when the total fits the entry capacity (an attempt
+__device__ __forceinline__ void bin_fill(int64_t i, const GRec* __restrict__ rec, const GaussGrid& G,
+                                         const int32_t* __restrict__ cell_start, int32_t* __restrict__ cell_cnt,
+                                         uint4* __restrict__ ent)
+{
+    const float4 r0 = rec[i].r0;
+    if (r0.w < 0.f) return;
+    const uint4 en = make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i);
+    int lo[3], hi[3];
+    cell_range(G, en, lo, hi);
+    for (int z = lo[2]; z <= hi[2]; ++z)
+        for (int y = lo[1]; y <= hi[1]; ++y)
+            for (int x = lo[0]; x <= hi[0]; ++x) {
+                const int c = (z * G.dims[1] + y) * G.dims[0] + x;
+                ent[cell_start[c] + atomicAdd(&cell_cnt[c], 1)] = en;
+            }
+}
+
+__global__ void bin_count_kernel(int64_t N, const GRec* __restrict__ rec, const GaussGrid* __restrict__ gridp,
+                                 int32_t* __restrict__ cell_cnt)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) bin_count(i, rec, *gridp, cell_cnt);
+}
+
+// After the scan of a binning attempt's counts: whether the cell lists fit
+// the entry capacity (the fill pass and later attempts read it; an attempt
 // after the first that fits marks the status word: the grid was coarsened).
-// After the count pass of a binning attempt: whether the cell lists fit the
-// entry capacity (the fill pass and later attempts read it).
 struct BinScanFinal {
     GaussGrid* grid;
     int64_t entries_cap;
@@ -309,26 +366,142 @@ __global__ void bin_fill_kernel(int64_t N, const GRec* __restrict__ rec, const G
                                 uint4* __restrict__ ent)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N || !gridp->fits) return;
-    const float4 r0 = rec[i].r0;
-    if (r0.w < 0.f) return;
-    const GaussGrid G = *gridp;
-    const uint4 en = make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i);
-    int lo[3], hi[3];
-    cell_range(G, en, lo, hi);
-    for (int z = lo[2]; z <= hi[2]; ++z)
-        for (int y = lo[1]; y <= hi[1]; ++y)
-            for (int x = lo[0]; x <= hi[0]; ++x) {
-                const int c = (z * G.dims[1] + y) * G.dims[0] + x;
-                const int pos = cell_start[c] + atomicAdd(&cell_cnt[c], 1);
-                ent[pos] = en;
-            }
+    if (i < N && gridp->fits) bin_fill(i, rec, *gridp, cell_start, cell_cnt, ent);
 }
 
-// Texel-centre directions, computed in fp64 and rounded once.
-__global__ void texel_dirs_kernel(int R, float4* __restrict__ dirs)
+// ---------------------------------------------------------------------------
+// Binning by one CTA. For small sets (kBinOneCta) it does all of it, records
+// included, with the cells counted in shared memory, where the general path's
+// seven launches are most of the time (2,000 Gaussians: a bake of 64 probes
+// 122 us with 22 launches, 77 us with 4; 24 us of it here, a third waiting
+// for the parameters); for larger ones it is the later attempts' launch,
+// which returns at once when the first grid fitted.
+// Attempts (decided on the device, no host read-back): the requested grid; if
+// its cell lists overflow the workspace, a grid with 1/16 of the cells; then
+// one of at most 2 cells, whose lists (at most 2 entries per Gaussian) always
+// fit, since the workspace holds at least 24 per Gaussian.
+// ---------------------------------------------------------------------------
+constexpr int64_t kBinOneCta = 4096;
+
+struct BinK {
+    sop_gaussians g;
+    float alpha_min;
+    int64_t caps[kBinAttempts];
+    int64_t entries_cap;
+    GRec* rec;
+    GaussGrid* grid;
+    int32_t *bbox, *cell_start, *cell_cnt;
+    uint4* ent;
+    unsigned int* status;
+    int32_t first;  // 0: every attempt; 1: those after the first
+    int32_t prep;   // compute the records and the box too
+};
+
+constexpr int kBinSmemCells = 8192;  // cells counted in shared memory
+
+// f(cell, entry) for the cells of the CTA's Gaussians
+template <class F>
+__device__ __forceinline__ void bin_visit(int64_t n, const GRec* __restrict__ rec, const GaussGrid& G, F f)
+{
+    for (int64_t i = threadIdx.x; i < n; i += 1024) {
+        const float4 r0 = rec[i].r0;
+        if (r0.w < 0.f) continue;
+        const uint4 en = make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i);
+        int lo[3], hi[3];
+        cell_range(G, en, lo, hi);
+        for (int z = lo[2]; z <= hi[2]; ++z)
+            for (int y = lo[1]; y <= hi[1]; ++y)
+                for (int x = lo[0]; x <= hi[0]; ++x) f((z * G.dims[1] + y) * G.dims[0] + x, en);
+    }
+}
+
+__global__ void __launch_bounds__(1024) bin_one_kernel(const BinK k)
+{
+    __shared__ int32_t s_box[6][32];
+    __shared__ long long s_w[kScanThreads / 32];
+    __shared__ GaussGrid G;
+    __shared__ long long s_tot;
+    __shared__ int32_t s_cnt[kBinSmemCells];
+    const int tid = threadIdx.x;
+    if (k.first > 0 && k.grid->fits) return;
+    if (k.prep) {
+        float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+        for (int64_t i = tid; i < k.g.n; i += 1024) gauss_record(k.g, i, k.alpha_min, k.rec, k.status, lo, hi);
+        int32_t box[6];
+        cta_box(lo, hi, s_box, box);
+        if (tid == 0)
+            for (int a = 0; a < 6; ++a) k.bbox[a] = box[a];
+    }
+    __syncthreads();
+    bool in_smem = false;
+    for (int level = k.first; level < kBinAttempts; ++level) {
+        if (tid == 0) {
+            int32_t box[6];
+            for (int a = 0; a < 6; ++a) box[a] = k.bbox[a];
+            G = grid_geometry(box, k.caps[level], level);
+            s_tot = 0;
+        }
+        __syncthreads();
+        const int nc = G.ncells;
+        in_smem = nc <= kBinSmemCells;
+        int32_t* cnt = in_smem ? s_cnt : k.cell_cnt;
+        for (int c = tid; c < nc; c += 1024) cnt[c] = 0;
+        __syncthreads();
+        bin_visit(k.g.n, k.rec, G, [&](int c, const uint4&) { atomicAdd(cnt + c, 1); });
+        __syncthreads();
+        // exclusive scan of the counts, a tile of them at a time; in shared
+        // memory they become the fill's cursors, else they are cleared
+        for (int c0 = 0; c0 < nc; c0 += kScanTile) {
+            int32_t v[kScanPer];
+            long long sum = 0, tot;
+#pragma unroll
+            for (int e = 0; e < kScanPer; ++e) {
+                const int c = c0 + tid * kScanPer + e;
+                v[e] = c >= nc ? 0 : (in_smem ? s_cnt[c] : __ldcg(k.cell_cnt + c));  // (counted by atomics in L2)
+                sum += v[e];
+            }
+            long long run = scan_block_inclusive(sum, s_w, &tot) - sum + s_tot;
+#pragma unroll
+            for (int e = 0; e < kScanPer; ++e) {
+                const int c = c0 + tid * kScanPer + e;
+                if (c < nc) {
+                    const int32_t at = (int32_t)(run < INT32_MAX ? run : INT32_MAX);
+                    k.cell_start[c] = at;
+                    cnt[c] = in_smem ? at : 0;
+                }
+                run += v[e];
+            }
+            __syncthreads();
+            if (tid == 0) s_tot += tot;
+            __syncthreads();
+        }
+        if (tid == 0) {
+            k.cell_start[nc] = (int32_t)(s_tot < INT32_MAX ? s_tot : INT32_MAX);
+            BinScanFinal{&G, k.entries_cap, k.status}(s_tot);
+            *k.grid = G;
+        }
+        __syncthreads();
+        if (G.fits) break;
+    }
+    if (!G.fits) return;
+    if (!k.ent) {  // a launch of its own fills, with cleared counters
+        if (in_smem)
+            for (int c = tid; c < G.ncells; c += 1024) k.cell_cnt[c] = 0;
+    } else if (in_smem) {
+        bin_visit(k.g.n, k.rec, G, [&](int c, const uint4& en) { k.ent[atomicAdd(s_cnt + c, 1)] = en; });
+    } else {
+        bin_visit(k.g.n, k.rec, G, [&](int c, const uint4& en) {
+            k.ent[k.cell_start[c] + atomicAdd(k.cell_cnt + c, 1)] = en;
+        });
+    }
+}
+
+// Start of a bake's trace: the counters cleared, and the texel-centre
+// directions, computed in fp64 and rounded once.
+__global__ void trace_begin_kernel(int R, float4* __restrict__ dirs, unsigned long long* __restrict__ stats)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < 8) stats[t] = 0ull;
     if (t >= R * R) return;
     double d[3];
     oct_decode_centre_f64(R, t % R, t / R, d);
@@ -1038,49 +1211,69 @@ __global__ void __launch_bounds__(256, OUT == kTraceAtlas ? 4 : 3) trace_kernel(
     }
 }
 
+static BinK bin_args(const sop_gaussians& g, float alpha_min, const BakeLayout& L, char* ws)
+{
+    BinK k;
+    k.g = g;
+    k.alpha_min = alpha_min;
+    k.caps[0] = L.cells_cap;
+    k.caps[1] = L.cells_cap / 16 > 64 ? L.cells_cap / 16 : 64;
+    k.caps[2] = 2;
+    k.entries_cap = L.entries_cap;
+    k.rec = reinterpret_cast<GRec*>(ws + L.rec);
+    k.grid = reinterpret_cast<GaussGrid*>(ws + L.hdr);
+    k.bbox = reinterpret_cast<int32_t*>(ws + L.bbox);
+    k.cell_start = reinterpret_cast<int32_t*>(ws + L.cell_start);
+    k.cell_cnt = reinterpret_cast<int32_t*>(ws + L.cell_cnt);
+    k.ent = reinterpret_cast<uint4*>(ws + L.ent);
+    k.status = status_word();
+    k.first = 0;
+    k.prep = 1;
+    return k;
+}
+
 cudaError_t launch_bake_bin(const sop_gaussians& g, float alpha_min, const BakeLayout& L, char* ws, cudaStream_t s)
 {
+    if (g.n <= kBinOneCta) {
+        bin_one_kernel<<<1, 1024, 0, s>>>(bin_args(g, alpha_min, L, ws));
+        return cudaGetLastError();
+    }
     const cudaError_t e = launch_bake_prep(g, alpha_min, L, ws, s);
     return e != cudaSuccess ? e : launch_bake_grid(g, L, ws, s);
 }
 
+// CTAs of gauss_prep_kernel; their boxes wait in the entries' space
+static unsigned prep_parts(int64_t n) { return (unsigned)((n + 255) / 256); }
+
 cudaError_t launch_bake_prep(const sop_gaussians& g, float alpha_min, const BakeLayout& L, char* ws, cudaStream_t s)
 {
-    int32_t* bbox = reinterpret_cast<int32_t*>(ws + L.bbox);
-    GRec* rec = reinterpret_cast<GRec*>(ws + L.rec);
-    bbox_init_kernel<<<1, 32, 0, s>>>(bbox);
-    const unsigned nb = (unsigned)((g.n + 255) / 256);
-    if (g.n > 0) gauss_prep_kernel<<<nb, 256, 0, s>>>(g, alpha_min, rec, bbox, status_word());
+    if (g.n > 0)
+        gauss_prep_kernel<<<prep_parts(g.n), 256, 0, s>>>(g, alpha_min, reinterpret_cast<GRec*>(ws + L.rec),
+                                                          reinterpret_cast<int32_t*>(ws + L.ent),
+                                                          reinterpret_cast<int32_t*>(ws + L.cell_cnt), L.cells_cap,
+                                                          status_word());
     return cudaGetLastError();
 }
 
 cudaError_t launch_bake_grid(const sop_gaussians& g, const BakeLayout& L, char* ws, cudaStream_t s)
 {
-    GaussGrid* grid = reinterpret_cast<GaussGrid*>(ws + L.hdr);
-    int32_t* bbox = reinterpret_cast<int32_t*>(ws + L.bbox);
-    GRec* rec = reinterpret_cast<GRec*>(ws + L.rec);
-    int32_t* cstart = reinterpret_cast<int32_t*>(ws + L.cell_start);
-    int32_t* ccnt = reinterpret_cast<int32_t*>(ws + L.cell_cnt);
-    unsigned int* status = status_word();
-    const int bs = 256;
-    const unsigned nb = (unsigned)((g.n + bs - 1) / bs);
-    // Binning attempts, decided on the device (no host read-back): the
-    // requested grid; if its cell lists overflow the workspace, a grid with
-    // 1/16 of the cells; then one of at most 2 cells, whose lists (at most
-    // 2 entries per Gaussian) always fit, since the workspace holds at least
-    // 24 per Gaussian. Attempts after a fitting one return at once.
-    const int64_t caps[kBinAttempts] = {L.cells_cap, L.cells_cap / 16 > 64 ? L.cells_cap / 16 : 64, 2};
-    for (int a = 0; a < kBinAttempts; ++a) {
-        grid_setup_kernel<<<1, 1024, 0, s>>>(bbox, caps[a], a, grid, ccnt);
-        if (g.n > 0) bin_count_kernel<<<nb, bs, 0, s>>>(g.n, rec, grid, ccnt);
-        ScanArgs sa;
-        sa.n = &grid->ncells;
-        sa.skip = &grid->fits;
-        sa.cnt = ccnt;
-        sa.start = cstart;
-        sa.scratch = reinterpret_cast<long long*>(ws + L.scan);
-        launch_scan(sa, caps[a], BinScanFinal{grid, L.entries_cap, status}, s);
-    }
+    BinK k = bin_args(g, 0.f, L, ws);
+    const unsigned nb = (unsigned)((g.n + 255) / 256);
+    grid_setup_kernel<<<1, 1024, 0, s>>>(reinterpret_cast<const int32_t*>(ws + L.ent), (int32_t)prep_parts(g.n),
+                                         k.caps[0], k.bbox, k.grid);
+    if (g.n > 0) bin_count_kernel<<<nb, 256, 0, s>>>(g.n, k.rec, k.grid, k.cell_cnt);
+    ScanArgs sa;
+    sa.n = &k.grid->ncells;
+    sa.cnt = k.cell_cnt;
+    sa.start = k.cell_start;
+    sa.scratch = reinterpret_cast<long long*>(ws + L.scan);
+    launch_scan(sa, k.caps[0], BinScanFinal{k.grid, L.entries_cap, k.status}, s);
+    uint4* ent = k.ent;
+    k.first = 1;
+    k.prep = 0;
+    k.ent = nullptr;
+    bin_one_kernel<<<1, 1024, 0, s>>>(k);
+    if (g.n > 0) bin_fill_kernel<<<nb, 256, 0, s>>>(g.n, k.rec, k.grid, k.cell_start, k.cell_cnt, ent);
     return cudaGetLastError();
 }
 
@@ -1127,19 +1320,6 @@ __global__ void trace_status_kernel(const unsigned long long* stats, unsigned in
     if (status && (stats[3] & 1ull)) atomicOr(status, SOP_DEVSTAT_BAKE_TRUNCATED);
 }
 
-cudaError_t launch_bake_fill(const sop_gaussians& g, const BakeLayout& L, char* ws, cudaStream_t s)
-{
-    GaussGrid* grid = reinterpret_cast<GaussGrid*>(ws + L.hdr);
-    GRec* rec = reinterpret_cast<GRec*>(ws + L.rec);
-    int32_t* cstart = reinterpret_cast<int32_t*>(ws + L.cell_start);
-    int32_t* ccnt = reinterpret_cast<int32_t*>(ws + L.cell_cnt);
-    uint4* ent = reinterpret_cast<uint4*>(ws + L.ent);
-    const int bs = 256;
-    if (g.n > 0)
-        bin_fill_kernel<<<(unsigned)((g.n + bs - 1) / bs), bs, 0, s>>>(g.n, rec, grid, cstart, ccnt, ent);
-    return cudaGetLastError();
-}
-
 // persistent grid: as many CTAs as fit on the device at once (fewer for a
 // small launch)
 template <int OUT>
@@ -1164,8 +1344,7 @@ cudaError_t launch_bake_trace(const sop_atlas& atlas, const sop_bake_params& bp,
     const int R = atlas.R;
     float4* dirs = reinterpret_cast<float4*>(ws + L.dirs);
     unsigned long long* stats = reinterpret_cast<unsigned long long*>(ws + L.stats);
-    trace_reset_kernel<<<1, 32, 0, s>>>(stats);
-    texel_dirs_kernel<<<(R * R + 127) / 128, 128, 0, s>>>(R, dirs);
+    trace_begin_kernel<<<(R * R + 127) / 128, 128, 0, s>>>(R, dirs, stats);
     TraceK k;
     k.rec = reinterpret_cast<GRec*>(ws + L.rec);
     k.grid = grid;

@@ -575,7 +575,6 @@ cudaError_t launch_fps(const float* pts, const float* nrm, int64_t n, int32_t k,
         o = align256(o + 4 * (size_t)cells);
         ScanArgs sa;
         sa.n = mm + 6;
-        sa.skip = nullptr;
         sa.cnt = cnt;
         sa.start = reinterpret_cast<int32_t*>(ws + o);
         o = align256(o + 4 * (size_t)(cells + 1));

@@ -2097,7 +2097,6 @@ SitesGrid launch_sites_grid(const float* sites, int32_t N, char* ws, cudaStream_
         sites_count_kernel<<<nb, 256, 0, s>>>(sites, N, grid, ccnt);
         ScanArgs sa;
         sa.n = &grid->ncells;
-        sa.skip = nullptr;
         sa.cnt = ccnt;
         sa.start = cstart;
         sa.scratch = scan;

@@ -259,9 +259,7 @@ sop_status sop_bake_bin(const sop_gaussians* g, const sop_bake_params* params, v
     if ((st = bake_fit(g->n, params->grid_density, ws, ws_bytes, L)) != SOP_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     char* w = (char*)ws;
-    st = cuda_status(sop::launch_bake_bin(*g, params->alpha_min, L, w, s), "sop_bake_bin (binning)");
-    if (st != SOP_OK) return st;
-    return cuda_status(sop::launch_bake_fill(*g, L, w, s), "sop_bake_bin (fill)");
+    return cuda_status(sop::launch_bake_bin(*g, params->alpha_min, L, w, s), "sop_bake_bin");
 }
 
 sop_status sop_bake_trace(const sop_gaussians* g, const sop_atlas* atlas, const sop_bake_params* params, void* ws,
@@ -586,9 +584,8 @@ sop_status surr_feats_into(const sop_surrogate* net, const sop_gaussians* g, con
                            int32_t R, const sop_bake_params* bp, float* feats, int32_t* list, char* w,
                            const SurrRunLayout& L, cudaStream_t s, const char* what)
 {
-    sop_status st = cuda_status(sop::launch_bake_bin(*g, bp->alpha_min, L.B, w + L.bake, s), what);
-    if (st != SOP_OK) return st;
-    st = cuda_status(sop::launch_bake_fill(*g, L.B, w + L.bake, s), what);
+    // (the features read the records, not the bake's grid)
+    sop_status st = cuda_status(sop::launch_bake_prep(*g, bp->alpha_min, L.B, w + L.bake, s), what);
     if (st != SOP_OK) return st;
     return cuda_status(sop::surr_features(*g, probe_pos, P, R, net->r_near, bp->alpha_min, bp->alpha_max,
                                           w + L.bake + L.B.rec, feats, list, w + L.feat, s),
@@ -826,7 +823,6 @@ sop_status sop_surrogate_infer(const sop_surrogate* net, const sop_gaussians* g,
     // branch b: the binning grid, then the spot check's sample traced into
     // the workspace's atlas
     st = cuda_status(sop::launch_bake_grid(*g, L.B, w + L.bake, b), "sop_surrogate_infer (binning)");
-    if (st == SOP_OK) st = cuda_status(sop::launch_bake_fill(*g, L.B, w + L.bake, b), "sop_surrogate_infer (binning)");
     if (st == SOP_OK)
         st = cuda_status(sop::launch_spot_pick(seed, P, n_spot, out->probe_pos, ids, pos, b),
                          "sop_surrogate_infer (sample)");

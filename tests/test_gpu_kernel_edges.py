@@ -5,6 +5,8 @@ import numpy as np
 import pytest
 import torch
 
+from tests.tolerance import assert_close
+
 pytestmark = pytest.mark.gpu
 F = np.float32
 
@@ -187,3 +189,51 @@ def test_shadow_shared_integrals(sop, orc, M, dtype, K, S):
     want, _, _ = orc.query_shade(*args, mode=orc.MODE_SHADOW)
     sens = orc.query_shade_sensitivity(*args, mode=orc.MODE_SHADOW)
     assert np.all(np.abs(out[sel] - want) <= 1e-5 * np.maximum(np.abs(want), 1e-3 * np.abs(want).mean()) + sens)
+
+
+def _cloud(rng, n, needles):
+    s = np.exp(rng.uniform(np.log(0.002), np.log(0.01), (n, 3)))
+    if needles:
+        s[:, 0] = 0.3
+    q = rng.standard_normal((n, 4))
+    g = dict(mean=rng.uniform(-1, 1, (n, 3)), scale=s, quat=q / np.linalg.norm(q, axis=1, keepdims=True).clip(1e-9),
+             opacity=rng.uniform(0.1, 0.9, n), rgb=rng.uniform(0, 1, (n, 3)))
+    return {k: v.astype(F) for k, v in g.items()}
+
+
+@pytest.mark.parametrize("n", [0, 1, 33, 4096, 4097, 70_000])
+def test_bake_binning_sizes(sop, orc, n):
+    """Binning by one CTA (up to 4,096 Gaussians) and by many: the traced maps
+    against the oracle on rays whose hits are not within rounding of a
+    decision."""
+    rng = np.random.default_rng(n)
+    g, pp, R = _cloud(rng, n, False), rng.uniform(-1.2, 1.2, (3, 3)).astype(F), 4
+    at = sop.make_atlas(cuda(pp), R)
+    sop.bake({k: cuda(v) for k, v in g.items()}, at)
+    sop.device_status()
+    rgb, occ, dep = (t.cpu().numpy() for t in at.interior())
+    o_rgb, o_occ, o_dep, fl, sens = orc.bake(g, pp, R, with_sens=True)
+    ok = fl == 0
+    if ok.any():  # the FP32 bound, plus the rounding of the texel directions
+        assert_close(occ[ok], o_occ[ok], what="O", absolute=sens[..., 3][ok])
+        assert_close(rgb[ok], o_rgb[ok], what="L_in", absolute=sens[..., :3][ok])
+
+
+@pytest.mark.parametrize("n,needles", [(1000, False), (4096, False), (4096, True)])
+def test_bake_binning_paths_agree(sop, n, needles):
+    """The same Gaussians binned by one CTA and, with invisible ones added to
+    pass 4,096, by many: the same bits. Needles' boxes span so many cells that
+    their lists overflow the workspace and a coarser grid is taken (the status
+    word says so), in both."""
+    rng = np.random.default_rng(n)
+    g, pp = _cloud(rng, n, needles), rng.uniform(-1.2, 1.2, (5, 3)).astype(F)
+    extra = _cloud(rng, 4097 - n + 700, False)
+    extra["opacity"][:] = 1e-3
+    both = {k: np.concatenate([g[k], extra[k]]) for k in g}
+    out = []
+    for c in (g, both):
+        at = sop.make_atlas(cuda(pp), 8)
+        sop.bake({k: cuda(v) for k, v in c.items()}, at)
+        assert bool(sop.device_status() & sop.DEVSTAT_GRID_COARSENED) == needles
+        out.append((at.rgbo.cpu().numpy(), at.depth.cpu().numpy()))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
