@@ -937,13 +937,13 @@ static cudaError_t adjoint_tile_launch(const AdjK& k, cudaStream_t s)
 {
     const size_t smem = adj_smem(k.R, k.S, k.K).total;
     auto fn = adjoint_tile_kernel<DT>;
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kAdjPts * 32, smem);
     if (e != cudaSuccess) return e;
-    const int64_t tiles = (k.M + kAdjPts - 1) / kAdjPts, most = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+    // two CTAs an SM (their registers' limit) where shared memory holds both
+    const int64_t tiles = (k.M + kAdjPts - 1) / kAdjPts, most = (int64_t)sms * (smem <= 110 * 1024 ? 2 : 1);
     fn<<<(unsigned)(tiles < most ? tiles : most), kAdjPts * 32, smem, s>>>(k);
     return cudaGetLastError();
 }
@@ -994,8 +994,8 @@ cudaError_t launch_adjoint(const QueryArgs& a, const QueryLayout& L, char* ws, c
     k.perm = perm;
     k.genv4 = reinterpret_cast<float4*>(ws + L.genv4);
 
-    cudaError_t e = cudaMemsetAsync(bucket, 0, sizeof(int32_t) * (size_t)(a.P + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(k.genv4, 0, sizeof(float4) * (size_t)a.He * a.We, s);
+    // (the buckets and the environment gradient lie next to each other)
+    cudaError_t e = cudaMemsetAsync(bucket, 0, L.genv4 - L.bucket + sizeof(float4) * (size_t)a.He * a.We, s);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((a.M + 255) / 256);
     perm_count_kernel<<<nb, 256, 0, s>>>(k.idx, a.K, a.M, bucket);

@@ -180,19 +180,21 @@ def _ptr(t):
         raise ValueError("libsop takes CUDA tensors")
     if not t.is_contiguous():
         raise ValueError("libsop takes contiguous tensors")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()  # (an int: the entry points' argtypes make it a pointer)
 
 
 def _f32(t, shape=None):
-    if t.dtype != torch.float32:
+    if t.dtype is not torch.float32:
         raise TypeError(f"expected float32, got {t.dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"expected shape {tuple(shape)}, got {tuple(t.shape)}")
     return _ptr(t)
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the current device's current stream, as torch.cuda.current_stream() gives
+    # it, without making a Stream object (3 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ws(nbytes, device):
@@ -225,14 +227,9 @@ class Atlas:
         return self.rgbo.shape[1] - 2
 
     def c(self):
-        d = AtlasDesc()
-        d.rgbo = self.rgbo.data_ptr()
-        d.depth = self.depth.data_ptr() if self.depth is not None else None
-        d.rgbo_dtype, d.depth_dtype = self.rgbo_dtype, self.depth_dtype
-        d.P, d.R = self.P, self.R
-        d.depth_scale = self.depth_scale
-        d.probe_pos = self.probe_pos.data_ptr()
-        d.probe_nrm = self.probe_nrm.data_ptr() if self.probe_nrm is not None else None
+        d = AtlasDesc(self.rgbo.data_ptr(), None if self.depth is None else self.depth.data_ptr(), self.rgbo_dtype,
+                      self.depth_dtype, self.P, self.R, self.depth_scale, self.probe_pos.data_ptr(),
+                      None if self.probe_nrm is None else self.probe_nrm.data_ptr())
         self.desc = d
         return d
 
@@ -340,18 +337,10 @@ def read_bandwidth_gbs(nbytes, reps, device="cuda", trials=5):
 
 def _gauss(g):
     n = g["mean"].shape[0]
-    s = Gaussians()
-    s.mean = g["mean"].data_ptr() if n else None
-    s.scale = g["scale"].data_ptr() if n else None
-    s.quat = g["quat"].data_ptr() if n else None
-    s.opacity = g["opacity"].data_ptr() if n else None
-    s.rgb = g["rgb"].data_ptr() if n else None
-    s.n = n
-    for k, shp in (("mean", (n, 3)), ("scale", (n, 3)), ("quat", (n, 4)), ("opacity", (n,)), ("rgb", (n, 3))):
-        t = g[k]
-        if n:
-            _f32(t, shp)
-    return s
+    if not n:
+        return Gaussians(None, None, None, None, None, 0)
+    return Gaussians(_f32(g["mean"], (n, 3)), _f32(g["scale"], (n, 3)), _f32(g["quat"], (n, 4)),
+                     _f32(g["opacity"], (n,)), _f32(g["rgb"], (n, 3)), n)
 
 
 # ----------------------------------------------------------------------------
@@ -537,8 +526,10 @@ def bake(gauss, atlas: Atlas, t_near=0.0, alpha_min=1.0 / 255.0, alpha_max=0.99,
         if ws is None:
             _bake_ws.clear()
             ws = _bake_ws[(dev, n)] = BakeWorkspace(n, dev)
-    bake_bin(gauss, ws, t_near, alpha_min, alpha_max, t_stop)
-    bake_trace(gauss, atlas, ws, t_near, alpha_min, alpha_max, t_stop)
+    g = _gauss(gauss)
+    d = atlas.c()
+    bp = _bake_params(t_near, alpha_min, alpha_max, t_stop)
+    _check(load().sop_bake(C.byref(g), C.byref(d), C.byref(bp), _ptr(ws.buf), ws.buf.numel(), _stream()))
     return atlas
 
 
@@ -568,14 +559,13 @@ def query_shade(x, n, wo, albedo, rough, metal, atlas: Atlas, env, K, S, mode=MO
         out = torch.empty((M, 3), dtype=torch.float32, device=dev)
     idx = torch.empty((M, K), dtype=torch.int32, device=dev) if return_idx else None
     w = torch.empty((M, K), dtype=torch.float32, device=dev) if return_idx else None
-    need = int(lib.sop_query_workspace_bytes(C.byref(d), M, C.byref(sp), He, We))
-    ws = workspace if workspace is not None else _ws(need, dev)
-    for t, shp in ((x, (M, 3)), (n, (M, 3)), (wo, (M, 3)), (albedo, (M, 3)), (rough, (M,)), (metal, (M,)),
-                   (env, (He, We, 3))):
-        _f32(t, shp)
-    _check(lib.sop_query_shade(_ptr(x), _ptr(n), _ptr(wo), _ptr(albedo), _ptr(rough), _ptr(metal), M, C.byref(d),
-                               _ptr(env), He, We, dl,
-                               C.byref(sp), _ptr(out), _ptr(idx), _ptr(w), _ptr(ws), ws.numel(), _stream()))
+    ws = workspace
+    if ws is None:
+        ws = _ws(lib.sop_query_workspace_bytes(C.byref(d), M, C.byref(sp), He, We), dev)
+    v3, v1 = (M, 3), (M,)
+    _check(lib.sop_query_shade(_f32(x, v3), _f32(n, v3), _f32(wo, v3), _f32(albedo, v3), _f32(rough, v1),
+                               _f32(metal, v1), M, C.byref(d), _f32(env, (He, We, 3)), He, We, dl, C.byref(sp),
+                               _ptr(out), _ptr(idx), _ptr(w), _ptr(ws), ws.numel(), _stream()))
     if return_idx:
         return out, idx, w
     return out
@@ -602,8 +592,9 @@ def query_shade_backward(x, n, wo, albedo, rough, metal, atlas: Atlas, env, K, S
     _f32(grad_out, (M, 3))
     _f32(g["env"], (He, We, 3))
     _f32(g["maps"], (P, R, R, 4))
-    need = int(lib.sop_query_workspace_bytes(C.byref(d), M, C.byref(sp), He, We))
-    ws = workspace if workspace is not None else _ws(need, dev)
+    ws = workspace
+    if ws is None:
+        ws = _ws(lib.sop_query_workspace_bytes(C.byref(d), M, C.byref(sp), He, We), dev)
     _check(lib.sop_query_shade_backward(
         _ptr(x), _ptr(n), _ptr(wo), _ptr(albedo), _ptr(rough), _ptr(metal), M, C.byref(d), _ptr(env), He, We,
         None if dirs_local is None else _f32(dirs_local, (S, 3)), C.byref(sp), _ptr(grad_out), _ptr(g["albedo"]),
