@@ -33,7 +33,8 @@ namespace sop {
 //   r0 = (mu.xyz, rho)   rho < 0: never reaches alpha_min
 //   r1..r3 = M = diag(1/s) R^T row-major (9) then opacity
 //   r3.zw, r4.x = rgb; r4.yzw = half extents of the alpha_min ellipsoid's
-//   axis-aligned box (used to bin the Gaussian into grid cells)
+//   axis-aligned box (used to bin the Gaussian into grid cells; a G-buffer
+//   trace puts its surfel normal there)
 struct GRec {
     float4 r0, r1, r2, r3, r4;
 };
@@ -554,7 +555,8 @@ struct TraceK {
 
 // what a traced ray writes: the probe atlas texel (O, L_in, depth) or the
 // G-buffer entry (C, W, N, D, A, R, M)
-enum { kTraceAtlas = 0, kTraceGbuf = 1 };
+// (kTraceGbufN: the same with the surfel normals in the records' last words)
+enum { kTraceAtlas = 0, kTraceGbuf = 1, kTraceGbufN = 2 };
 
 constexpr int kWarpsPerCta = 8;
 constexpr int kHitCap = 256;  // per-warp hit buffer (shared memory)
@@ -579,9 +581,10 @@ struct RayAcc {
 
 // Unit normal of a Gaussian read as a surfel: its local axis of smallest
 // scale (the first of equal ones), a column of R(q).
-__device__ __forceinline__ float3 surfel_normal(const TraceK& k, const int32_t g)
+__device__ __forceinline__ float3 surfel_normal(const float* __restrict__ quat, const float* __restrict__ scale,
+                                                const int64_t g)
 {
-    const float sx = __ldg(k.scale + 3 * g), sy = __ldg(k.scale + 3 * g + 1), sz = __ldg(k.scale + 3 * g + 2);
+    const float sx = __ldg(scale + 3 * g), sy = __ldg(scale + 3 * g + 1), sz = __ldg(scale + 3 * g + 2);
     int am = 0;
     float sm = sx;
     if (sy < sm) {
@@ -589,8 +592,8 @@ __device__ __forceinline__ float3 surfel_normal(const TraceK& k, const int32_t g
         sm = sy;
     }
     if (sz < sm) am = 2;
-    const float qw = __ldg(k.quat + 4 * g), qx = __ldg(k.quat + 4 * g + 1), qy = __ldg(k.quat + 4 * g + 2),
-                qz = __ldg(k.quat + 4 * g + 3);
+    const float qw = __ldg(quat + 4 * g), qx = __ldg(quat + 4 * g + 1), qy = __ldg(quat + 4 * g + 2),
+                qz = __ldg(quat + 4 * g + 3);
     const float qn = sqrtf(qw * qw + qx * qx + qy * qy + qz * qz);
     const float w = qw / qn, x = qx / qn, y = qy / qn, z = qz / qn;
     if (am == 0) return f3(1.f - 2.f * (y * y + z * z), 2.f * (x * y + w * z), 2.f * (x * z - w * y));
@@ -659,120 +662,91 @@ __device__ __forceinline__ void eval_batch(const TraceK& k, const float3 o, cons
     }
 }
 
-// Sorts key/alp[0, n) (n <= kHitCap) by key: ranks for a few hits, a bitonic
-// network over the lanes up to 32, a shared-memory bitonic network above.
-__device__ __forceinline__ void sort_hits(uint64_t* key, float* alp, const int n, const int lane)
+// Sorts key/alp[0, n) (n <= kHitCap) by key: a bitonic network in shared memory.
+__device__ __noinline__ void sort_hits(uint64_t* key, float* alp, const int n, const int lane)
 {
     __syncwarp();
-    if (n > 32 && n <= 64) {
-        // 64 elements in registers, two a lane: element lane (a) and
-        // lane + 32 (b); a bitonic network whose j = 32 steps compare a lane's
-        // own pair and whose others exchange over the lanes
-        uint64_t ka = key[lane], kb = lane + 32 < n ? key[lane + 32] : ~0ull;
-        float aa = alp[lane], ab = lane + 32 < n ? alp[lane + 32] : 0.f;
-#pragma unroll 1
-        for (int kk = 2; kk <= 64; kk <<= 1) {
-#pragma unroll 1
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                if (j == 32) {
-                    // (kk = 64: every pair ascending)
-                    if (kb < ka) {
-                        const uint64_t tk = ka;
-                        ka = kb;
-                        kb = tk;
-                        const float ta = aa;
-                        aa = ab;
-                        ab = ta;
-                    }
-                    continue;
-                }
-                const bool lower = (lane & j) == 0;
-                // element index lane (+ 32): ascending where (index & kk) == 0
-                const bool up_a = (lane & kk) == 0;
-                const bool up_b = ((lane + 32) & kk) == 0;
-                const uint64_t koa = __shfl_xor_sync(0xffffffffu, ka, j);
-                const float aoa = __shfl_xor_sync(0xffffffffu, aa, j);
-                const uint64_t kob = __shfl_xor_sync(0xffffffffu, kb, j);
-                const float aob = __shfl_xor_sync(0xffffffffu, ab, j);
-                if ((lower == up_a) ? (koa < ka) : (koa > ka)) {
-                    ka = koa;
-                    aa = aoa;
-                }
-                if ((lower == up_b) ? (kob < kb) : (kob > kb)) {
-                    kb = kob;
-                    ab = aob;
-                }
-            }
-        }
-        key[lane] = ka;
-        alp[lane] = aa;
-        if (lane + 32 < n) {
-            key[lane + 32] = kb;
-            alp[lane + 32] = ab;
-        }
-    } else if (n > 64) {
-        int P2 = 64;
-        while (P2 < n) P2 <<= 1;
-        for (int i = n + lane; i < P2; i += 32) {
-            key[i] = ~0ull;
-            alp[i] = 0.f;
-        }
-        __syncwarp();
-        for (int kk = 2; kk <= P2; kk <<= 1) {
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                for (int i = lane; i < P2; i += 32) {
-                    const int ixj = i ^ j;
-                    if (ixj > i) {
-                        const uint64_t a = key[i], b = key[ixj];
-                        const bool up = (i & kk) == 0;
-                        if ((a > b) == up) {
-                            key[i] = b;
-                            key[ixj] = a;
-                            const float ta = alp[i];
-                            alp[i] = alp[ixj];
-                            alp[ixj] = ta;
-                        }
-                    }
-                }
-                __syncwarp();
-            }
-        }
-    } else if (n > 1 && n <= 12) {
-        // each lane's rank is the number of smaller keys
-        const uint64_t kv = lane < n ? key[lane] : ~0ull;
-        const float av = lane < n ? alp[lane] : 0.f;
-        int rank = 0;
-        for (int j = 0; j < n; ++j) rank += __shfl_sync(0xffffffffu, kv, j) < kv ? 1 : 0;
-        __syncwarp();
-        if (lane < n) {
-            key[rank] = kv;
-            alp[rank] = av;
-        }
-    } else if (n > 1) {
-        uint64_t kv = lane < n ? key[lane] : ~0ull;
-        float av = lane < n ? alp[lane] : 0.f;
-#pragma unroll
-        for (int kk = 2; kk <= 32; kk <<= 1) {
-#pragma unroll
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                const uint64_t ko = __shfl_xor_sync(0xffffffffu, kv, j);
-                const float ao = __shfl_xor_sync(0xffffffffu, av, j);
-                const bool lower = (lane & j) == 0;
-                const bool up = (lane & kk) == 0;
-                // keep the smaller key on the lower lane of an ascending pair
-                const bool tk = (lower == up) ? (ko < kv) : (ko > kv);
-                if (tk) {
-                    kv = ko;
-                    av = ao;
-                }
-            }
-        }
-        if (lane < n) {
-            key[lane] = kv;
-            alp[lane] = av;
-        }
+    int P2 = 64;
+    while (P2 < n) P2 <<= 1;
+    for (int i = n + lane; i < P2; i += 32) {
+        key[i] = ~0ull;
+        alp[i] = 0.f;
     }
     __syncwarp();
+    for (int kk = 2; kk <= P2; kk <<= 1) {
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            for (int i = lane; i < P2; i += 32) {
+                const int ixj = i ^ j;
+                if (ixj > i) {
+                    const uint64_t a = key[i], b = key[ixj];
+                    const bool up = (i & kk) == 0;
+                    if ((a > b) == up) {
+                        key[i] = b;
+                        key[ixj] = a;
+                        const float ta = alp[i];
+                        alp[i] = alp[ixj];
+                        alp[ixj] = ta;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// One step of a bitonic network over the lanes on (t, place) pairs.
+__device__ __forceinline__ void lane_step(uint32_t& t, uint32_t& p, const int j, const bool up, const int lane)
+{
+    const uint32_t ot = __shfl_xor_sync(0xffffffffu, t, j), op = __shfl_xor_sync(0xffffffffu, p, j);
+    const bool low = ((lane & j) == 0) == up;
+    const uint32_t nt = low ? min(t, ot) : max(t, ot);
+    p = nt == t ? p : op;
+    t = nt;
+}
+
+// The places of the n <= 64 hits of key[] in order of t*, alone (the upper
+// half of a key; 0xffffffff pads): lane l's hits are the l-th (pa) and, for
+// n > 32, the l + 32-nd (pb). Half the words of the keys move through the
+// network, and the hits themselves stay where they are. Returns false where
+// two t* are equal, whose order the Gaussians' indices decide.
+__device__ __forceinline__ bool order_hits(const uint64_t* key, const int n, const int lane, uint32_t& ta, uint32_t& pa,
+                                           uint32_t& tb, uint32_t& pb)
+{
+    const unsigned full = 0xffffffffu;
+    ta = lane < n ? (uint32_t)(key[lane] >> 32) : 0xffffffffu;
+    pa = lane;
+    tb = 0xffffffffu;
+    pb = lane + 32;
+    if (n <= 32) {
+#pragma unroll
+        for (int kk = 2; kk <= 32; kk <<= 1) {
+            if (kk > 8 && n <= kk / 2) break;  // the rest are pads
+#pragma unroll
+            for (int j = kk >> 1; j > 0; j >>= 1) lane_step(ta, pa, j, (lane & kk) == 0, lane);
+        }
+        const uint32_t before = __shfl_up_sync(full, ta, 1);
+        return !__any_sync(full, lane > 0 && lane < n && before == ta);
+    }
+    tb = lane + 32 < n ? (uint32_t)(key[lane + 32] >> 32) : 0xffffffffu;
+#pragma unroll 1
+    for (int kk = 2; kk <= 64; kk <<= 1)
+#pragma unroll 1
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            if (j == 32) {  // (kk = 64) a lane's own pair
+                const bool sw = tb < ta;
+                const uint32_t t = ta, p = pa;
+                ta = sw ? tb : ta;
+                pa = sw ? pb : pa;
+                tb = sw ? t : tb;
+                pb = sw ? p : pb;
+                continue;
+            }
+            // element index lane (+ 32): ascending where (index & kk) == 0
+            lane_step(ta, pa, j, (lane & kk) == 0, lane);
+            lane_step(tb, pb, j, ((lane + 32) & kk) == 0, lane);
+        }
+    const uint32_t ba = __shfl_up_sync(full, ta, 1), bl = __shfl_sync(full, ta, 31), bu = __shfl_up_sync(full, tb, 1);
+    return !__any_sync(full, (lane > 0 && ba == ta) || (lane + 32 < n && (lane > 0 ? bu : bl) == tb));
 }
 
 // Composites the hits with t* < thr (every hit when `all`). They move to the
@@ -814,14 +788,18 @@ __device__ __forceinline__ void composite_hits(const TraceK& k, uint64_t* key, f
     }
     n = nr;
     if (nd == 0) return;
-    sort_hits(dkey, dalp, nd, lane);
+    uint32_t ta, pa, tb, pb;
+    bool places = false;  // the hits stay in place and pa, pb say their order
+    if (nd <= 64) places = order_hits(dkey, nd, lane, ta, pa, tb, pb);
+    if (!places) sort_hits(dkey, dalp, nd, lane);
     int used = 0;
     for (int cb = 0; cb < nd && !acc.done; cb += 32) {
         const int h = cb + lane;
         const bool on = h < nd;
-        const uint64_t kh = on ? dkey[h] : 0ull;
+        const uint32_t at = places ? (cb == 0 ? pa : pb) : (uint32_t)h;
+        const uint64_t kh = on ? dkey[at] : 0ull;
         const float th_hit = o2f((int32_t)((uint32_t)(kh >> 32) ^ 0x80000000u));
-        const float a = on ? dalp[h] : 0.f;
+        const float a = on ? dalp[at] : 0.f;
         const int32_t gh = (int32_t)(uint32_t)(kh & 0xffffffffu);
         // inclusive prefix product of (1 - alpha)
         float pin = 1.f - a;
@@ -845,8 +823,8 @@ __device__ __forceinline__ void composite_hits(const TraceK& k, uint64_t* key, f
             acc.L2 = fmaf(w, r4.x, acc.L2);
             acc.Dacc = fmaf(w, th_hit, acc.Dacc);
             acc.Wacc += w;
-            if (OUT == kTraceGbuf) {
-                const float3 nv = surfel_normal(k, gh);
+            if (OUT != kTraceAtlas) {
+                const float3 nv = OUT == kTraceGbufN ? f3(r4.y, r4.z, r4.w) : surfel_normal(k.quat, k.scale, gh);
                 const float ws = dot3(nv, d) > 0.f ? -w : w;
                 acc.N0 = fmaf(ws, nv.x, acc.N0);
                 acc.N1 = fmaf(ws, nv.y, acc.N1);
@@ -941,7 +919,7 @@ constexpr int kCompositeAt = 48;
 // composite the queue is always empty, so the set of hits composited, and
 // with it every rounding, is the same on every run.
 template <int OUT>
-__global__ void __launch_bounds__(256, OUT == kTraceAtlas ? 4 : 3) trace_kernel(const TraceK k)
+__global__ void __launch_bounds__(256, 4) trace_kernel(const TraceK k)
 {
     __shared__ uint64_t s_key[kWarpsPerCta][kHitCap];
     __shared__ float s_alpha[kWarpsPerCta][kHitCap];
@@ -1162,7 +1140,7 @@ __global__ void __launch_bounds__(256, OUT == kTraceAtlas ? 4 : 3) trace_kernel(
         Dacc += __shfl_xor_sync(0xffffffffu, Dacc, off);
         Wacc += __shfl_xor_sync(0xffffffffu, Wacc, off);
     }
-    if (OUT == kTraceGbuf) {
+    if (OUT != kTraceAtlas) {
         float v[8] = {acc.N0, acc.N1, acc.N2, acc.A0, acc.A1, acc.A2, acc.Rg, acc.Mg};
 #pragma unroll
         for (int c = 0; c < 8; ++c)
@@ -1314,6 +1292,19 @@ __global__ void trace_reset_kernel(unsigned long long* stats)
     if (threadIdx.x < 8) stats[threadIdx.x] = 0ull;
 }
 
+// The surfel normals into the records' last three words, where binning, now
+// done, had the box's half extents.
+__global__ void gbuf_normals_kernel(int64_t n, const float* __restrict__ quat, const float* __restrict__ scale,
+                                    GRec* __restrict__ rec)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float3 v = surfel_normal(quat, scale, i);
+    rec[i].r4.y = v.x;
+    rec[i].r4.z = v.y;
+    rec[i].r4.w = v.z;
+}
+
 // the truncation bit of a G-buffer trace into the status word
 __global__ void trace_status_kernel(const unsigned long long* stats, unsigned int* status)
 {
@@ -1412,7 +1403,16 @@ cudaError_t launch_trace_gbuffer(const sop_gaussians& g, const float* albedo, co
     k.run_if = nullptr;
     const int64_t rays = (int64_t)n_origins * n_dirs;
     if (rays == 0) return cudaGetLastError();
-    trace_kernel<kTraceGbuf><<<trace_blocks<kTraceGbuf>(rays), kWarpsPerCta * 32, 0, s>>>(k);
+    // A normal is 7 loads and some 90 instructions a composited hit, or one
+    // pass over the Gaussians: the pass where there are rays enough (2.07M
+    // rays through 1M surfels: GBUF_OLD -> GBUF_NEW us)
+    if (g.n > 0 && 2 * rays >= g.n) {
+        gbuf_normals_kernel<<<(unsigned)((g.n + 255) / 256), 256, 0, s>>>(g.n, g.quat, g.scale,
+                                                                          reinterpret_cast<GRec*>(ws + L.rec));
+        trace_kernel<kTraceGbufN><<<trace_blocks<kTraceGbufN>(rays), kWarpsPerCta * 32, 0, s>>>(k);
+    } else {
+        trace_kernel<kTraceGbuf><<<trace_blocks<kTraceGbuf>(rays), kWarpsPerCta * 32, 0, s>>>(k);
+    }
     trace_status_kernel<<<1, 1, 0, s>>>(stats, k.status);
     return cudaGetLastError();
 }
