@@ -33,7 +33,8 @@ namespace sop {
 //   r0 = (mu.xyz, rho)   rho < 0: never reaches alpha_min
 //   r1..r3 = M = diag(1/s) R^T row-major (9) then opacity
 //   r3.zw, r4.x = rgb; r4.yzw = half extents of the alpha_min ellipsoid's
-//   axis-aligned box (used to bin the Gaussian into grid cells)
+//   axis-aligned box (used to bin the Gaussian into grid cells; a G-buffer
+//   trace puts its surfel normal there)
 struct GRec {
     float4 r0, r1, r2, r3, r4;
 };
@@ -554,7 +555,8 @@ struct TraceK {
 
 // what a traced ray writes: the probe atlas texel (O, L_in, depth) or the
 // G-buffer entry (C, W, N, D, A, R, M)
-enum { kTraceAtlas = 0, kTraceGbuf = 1 };
+// (kTraceGbufN: the same with the surfel normals in the records' last words)
+enum { kTraceAtlas = 0, kTraceGbuf = 1, kTraceGbufN = 2 };
 
 constexpr int kWarpsPerCta = 8;
 constexpr int kHitCap = 256;  // per-warp hit buffer (shared memory)
@@ -824,7 +826,7 @@ __device__ __forceinline__ void composite_hits(const TraceK& k, uint64_t* key, f
             acc.Dacc = fmaf(w, th_hit, acc.Dacc);
             acc.Wacc += w;
             if (OUT != kTraceAtlas) {
-                const float3 nv = surfel_normal(k.quat, k.scale, gh);
+                const float3 nv = OUT == kTraceGbufN ? f3(r4.y, r4.z, r4.w) : surfel_normal(k.quat, k.scale, gh);
                 const float ws = dot3(nv, d) > 0.f ? -w : w;
                 acc.N0 = fmaf(ws, nv.x, acc.N0);
                 acc.N1 = fmaf(ws, nv.y, acc.N1);
@@ -1292,6 +1294,19 @@ __global__ void trace_reset_kernel(unsigned long long* stats)
     if (threadIdx.x < 8) stats[threadIdx.x] = 0ull;
 }
 
+// The surfel normals into the records' last three words, where binning, now
+// done, had the box's half extents.
+__global__ void gbuf_normals_kernel(int64_t n, const float* __restrict__ quat, const float* __restrict__ scale,
+                                    GRec* __restrict__ rec)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float3 v = surfel_normal(quat, scale, i);
+    rec[i].r4.y = v.x;
+    rec[i].r4.z = v.y;
+    rec[i].r4.w = v.z;
+}
+
 // the truncation bit of a G-buffer trace into the status word
 __global__ void trace_status_kernel(const unsigned long long* stats, unsigned int* status)
 {
@@ -1390,7 +1405,16 @@ cudaError_t launch_trace_gbuffer(const sop_gaussians& g, const float* albedo, co
     k.run_if = nullptr;
     const int64_t rays = (int64_t)n_origins * n_dirs;
     if (rays == 0) return cudaGetLastError();
-    trace_kernel<kTraceGbuf><<<trace_blocks<kTraceGbuf>(rays), kWarpsPerCta * 32, 0, s>>>(k);
+    // A normal is 7 loads and some 90 instructions a composited hit, or one
+    // pass over the Gaussians: the pass where there are rays enough (2.07M
+    // rays through 1M surfels: 5,530 -> 5,315 us)
+    if (g.n > 0 && 2 * rays >= g.n) {
+        gbuf_normals_kernel<<<(unsigned)((g.n + 255) / 256), 256, 0, s>>>(g.n, g.quat, g.scale,
+                                                                          reinterpret_cast<GRec*>(ws + L.rec));
+        trace_kernel<kTraceGbufN><<<trace_blocks<kTraceGbufN>(rays), kWarpsPerCta * 32, 0, s>>>(k);
+    } else {
+        trace_kernel<kTraceGbuf><<<trace_blocks<kTraceGbuf>(rays), kWarpsPerCta * 32, 0, s>>>(k);
+    }
     trace_status_kernel<<<1, 1, 0, s>>>(stats, k.status);
     return cudaGetLastError();
 }
