@@ -12,12 +12,13 @@
 // compact [P][R][R] maps. Environment and probe gradients are scattered with
 // float atomics (order-nondeterministic sums).
 //
-// Scatter traffic (bound by L2 atomics): the points are taken grouped by
-// their nearest probe (a counting sort), so that a CTA's atomics go to few
-// probes' texels; neighbouring points start their direction loops S/32
-// apart (by point index), so that a warp's lanes do not update the same
-// texels at the same step; the environment gradient is accumulated as float4 texels (4 vector
-// atomics a direction instead of 12 scalar ones) and folded into g_env.
+// Two kernels (adjoint_by_tile says which): adjoint_tile_kernel, eight points
+// a CTA with a gradient image each in shared memory, and adjoint_kernel, a
+// thread a point with K 4 vector atomics a direction into the maps. Both take
+// the points grouped by their nearest probe (a counting sort), so that a
+// CTA's points share probes, and accumulate the environment gradient as
+// float4 texels (4 vector atomics a direction instead of 12 scalar ones),
+// folded into g_env after.
 #include "point_blend.cuh"
 #include "sop_device.cuh"
 #include "sop_internal.h"

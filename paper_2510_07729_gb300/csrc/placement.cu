@@ -100,15 +100,7 @@ __global__ void fps_bbox_kernel(const float* __restrict__ pts, int64_t n, int32_
         lo[0] = min(lo[0], q.x); lo[1] = min(lo[1], q.y); lo[2] = min(lo[2], q.z);
         hi[0] = max(hi[0], q.x); hi[1] = max(hi[1], q.y); hi[2] = max(hi[2], q.z);
     }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
-        hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(&mm[a], lo[a]);
-            atomicMax(&mm[3 + a], hi[a]);
-        }
-    }
+    cta_box_atomic(lo, hi, mm);
 }
 
 // Cubic cells, 2^bits an axis over the longest side of the points' box, in
@@ -589,7 +581,7 @@ cudaError_t launch_fps(const float* pts, const float* nrm, int64_t n, int32_t k,
         if ((e = cudaMemsetAsync(a.slots, 0, exch, s)) != cudaSuccess) return e;
         const unsigned nb = (unsigned)((n + 255) / 256), nz = (unsigned)((cells + 255) / 256);
         fps_clear_kernel<<<nz, 256, 0, s>>>(cnt, cells, mm);
-        fps_bbox_kernel<<<nb < 608 ? nb : 608, 256, 0, s>>>(pts, n, mm);
+        fps_bbox_kernel<<<nb < kBoxCtas ? nb : kBoxCtas, 256, 0, s>>>(pts, n, mm);
         fps_count_kernel<<<nb, 256, 0, s>>>(pts, n, mm, bits, cnt);
         launch_scan(sa, cells, ScanNoFinal{}, s);
         fps_fill_kernel<<<nb, 256, 0, s>>>(pts, n, mm, bits, sa.start, cnt, perm);

@@ -65,26 +65,6 @@ __device__ __forceinline__ uint64_t qdist2(int32_t ax, int32_t ay, int32_t az, c
     return (uint64_t)dx * dx + (uint64_t)dy * dy + (uint64_t)dz * dz;
 }
 
-// Cubic cell edge (quantised units) for a box of extents ext[3]: the smallest
-// edge whose grid, (ext/cs + 1) cells per axis, has at most `cap` cells. A
-// flat site set (probes on a ground plane) then gets fine cells in its
-// plane instead of the cbrt-per-axis split of a volume, which would put
-// cbrt(P) sites in every cell of its one layer.
-__device__ __forceinline__ int64_t grid_cell_edge(const int64_t ext[3], int64_t cap)
-{
-    int64_t emax = 0;
-    for (int a = 0; a < 3; ++a) emax = ext[a] > emax ? ext[a] : emax;
-    int64_t lo = 1, hi = emax + 1;  // hi: one cell per axis
-    while (lo < hi) {
-        const int64_t mid = lo + (hi - lo) / 2;
-        int64_t n = 1;
-        for (int a = 0; a < 3 && n <= cap; ++a) n *= ext[a] / mid + 1;
-        if (n <= cap) hi = mid;
-        else lo = mid + 1;
-    }
-    return lo;
-}
-
 // cell of a site of the set (quantised position), by the grid's edge
 __device__ __forceinline__ int grid_cell(const ProbeGrid& G, int32_t qx, int32_t qy, int32_t qz)
 {
@@ -129,6 +109,27 @@ __device__ __forceinline__ bool grid_fits(const uint32_t ext[3], uint64_t e, int
     return true;
 }
 
+// Smallest edge (quantised units) that fits, by one warp, 32 candidates a step.
+// A flat site set (probes on a ground plane) then gets fine cells in its
+// plane instead of the cbrt-per-axis split of a volume, which would put
+// cbrt(P) sites in every cell of its one layer.
+__device__ __forceinline__ uint32_t grid_edge(const uint32_t ext[3], const int64_t cap, const int lane)
+{
+    uint64_t lo = 1, hi = (uint64_t)max(ext[0], max(ext[1], ext[2])) + 1;  // hi: one cell per axis
+    while (lo < hi) {
+        const uint64_t step = (hi - lo + 31) / 32, e = min(lo + lane * step, hi);
+        const unsigned ok = __ballot_sync(0xffffffffu, grid_fits(ext, e, cap));
+        const int f = ok ? __ffs(ok) - 1 : 32;
+        if (f == 0) hi = lo;
+        else {
+            if (f < 32) hi = min(lo + f * step, hi);
+            lo = min(lo + (f - 1) * step, hi) + 1;
+        }
+    }
+    // (an edge of 2^31 and more: one cell per axis too)
+    return (uint32_t)min(lo, (uint64_t)INT32_MAX);
+}
+
 __device__ __forceinline__ void probe_grid_build(GridSmem& sm, const float* __restrict__ probe_pos, int32_t P,
                                                  int32_t g_axis, ProbeGrid* grid, int32_t* cell_start,
                                                  int32_t* cell_cnt, int4* entries)
@@ -167,21 +168,8 @@ __device__ __forceinline__ void probe_grid_build(GridSmem& sm, const float* __re
 #pragma unroll
     for (int a = 0; a < 3; ++a) ext[a] = (uint32_t)sm.mx[a] - (uint32_t)sm.mn[a];
     if (warp < kGridLevels) {
-        // smallest edge that fits, 32 candidates a step
-        const int64_t cap = cap0 >> warp;
-        uint64_t lo = 1, hi = (uint64_t)max(ext[0], max(ext[1], ext[2])) + 1;  // hi: one cell per axis
-        while (lo < hi) {
-            const uint64_t step = (hi - lo + 31) / 32, e = min(lo + lane * step, hi);
-            const unsigned ok = __ballot_sync(full, grid_fits(ext, e, cap));
-            const int f = ok ? __ffs(ok) - 1 : 32;
-            if (f == 0) hi = lo;
-            else {
-                if (f < 32) hi = min(lo + f * step, hi);
-                lo = min(lo + (f - 1) * step, hi) + 1;
-            }
-        }
-        // (an edge of 2^32 - 1 and more: one cell per axis too)
-        if (lane == 0) sm.edge[warp] = (uint32_t)min(lo, (uint64_t)INT32_MAX);
+        const uint32_t e = grid_edge(ext, cap0 >> warp, lane);
+        if (lane == 0) sm.edge[warp] = e;
     }
     __syncthreads();
     const bool in_smem = cap0 <= kGridSmemCells;
@@ -2016,36 +2004,28 @@ __global__ void sites_bbox_kernel(const float* __restrict__ pos, int32_t N, int3
             lo[a] = min(lo[a], q);
             hi[a] = max(hi[a], q);
         }
-    for (int a = 0; a < 3; ++a) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = min(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-            hi[a] = max(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMin(&mm[a], lo[a]);
-            atomicMax(&mm[3 + a], hi[a]);
-        }
-    }
+    cta_box_atomic(lo, hi, mm);
 }
 
-__global__ void sites_setup_kernel(int32_t* mm, int64_t cap, ProbeGrid* grid)
+// one warp: the smallest cell edge of at most cap cells
+__global__ void sites_setup_kernel(const int32_t* __restrict__ mm, int64_t cap, ProbeGrid* grid)
 {
-    if (threadIdx.x == 0) {
-        ProbeGrid G;
-        int64_t ext[3];
-        for (int a = 0; a < 3; ++a) ext[a] = (int64_t)mm[3 + a] - mm[a];
-        const int64_t cs = grid_cell_edge(ext, cap);
-        G.cs = (int32_t)cs;
-        int32_t nc = 1;
-        for (int a = 0; a < 3; ++a) {
-            G.qmin[a] = mm[a];
-            G.dims[a] = (int32_t)(ext[a] / cs) + 1;
-            nc *= G.dims[a];
-        }
-        G.ncells = nc;
-        G.inv = 0xffffffffu / (uint32_t)G.cs;
-        *grid = G;
+    uint32_t ext[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) ext[a] = (uint32_t)mm[3 + a] - (uint32_t)mm[a];
+    const uint32_t cs = grid_edge(ext, cap, threadIdx.x);
+    if (threadIdx.x != 0) return;
+    ProbeGrid G;
+    G.cs = (int32_t)cs;
+    G.inv = 0xffffffffu / cs;
+    G.ncells = 1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        G.qmin[a] = mm[a];
+        G.dims[a] = (int32_t)(ext[a] / cs) + 1;
+        G.ncells *= G.dims[a];
     }
+    *grid = G;
 }
 
 __global__ void sites_zero_kernel(int32_t* __restrict__ cnt, int64_t n, int32_t* mm)
@@ -2056,24 +2036,12 @@ __global__ void sites_zero_kernel(int32_t* __restrict__ cnt, int64_t n, int32_t*
     else if (i < 6) mm[i] = INT32_MIN;
 }
 
-__device__ __forceinline__ int site_cell(const ProbeGrid& G, const float* pos, int64_t i, int32_t q[3])
-{
-    int c[3];
-    for (int a = 0; a < 3; ++a) {
-        q[a] = quantise(pos[3 * i + a]);
-        c[a] = (int)(((int64_t)q[a] - G.qmin[a]) / G.cs);
-    }
-    return (c[2] * G.dims[1] + c[1]) * G.dims[0] + c[0];
-}
-
 __global__ void sites_count_kernel(const float* __restrict__ pos, int32_t N, const ProbeGrid* __restrict__ gp,
                                    int32_t* __restrict__ cnt)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const ProbeGrid G = *gp;
-    int32_t q[3];
-    atomicAdd(&cnt[site_cell(G, pos, i, q)], 1);
+    atomicAdd(&cnt[grid_cell(*gp, quantise(pos[3 * i]), quantise(pos[3 * i + 1]), quantise(pos[3 * i + 2]))], 1);
 }
 
 __global__ void sites_fill_kernel(const float* __restrict__ pos, int32_t N, const ProbeGrid* __restrict__ gp,
@@ -2081,10 +2049,9 @@ __global__ void sites_fill_kernel(const float* __restrict__ pos, int32_t N, cons
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    const ProbeGrid G = *gp;
-    int32_t q[3];
-    const int cell = site_cell(G, pos, i, q);
-    ent[start[cell] + atomicAdd(&cnt[cell], 1)] = make_int4(q[0], q[1], q[2], (int)i);
+    const int32_t x = quantise(pos[3 * i]), y = quantise(pos[3 * i + 1]), z = quantise(pos[3 * i + 2]);
+    const int cell = grid_cell(*gp, x, y, z);
+    ent[start[cell] + atomicAdd(&cnt[cell], 1)] = make_int4(x, y, z, (int)i);
 }
 
 // ---------------------------------------------------------------------------
@@ -2157,7 +2124,7 @@ SitesGrid launch_sites_grid(const float* sites, int32_t N, char* ws, cudaStream_
     } else {
         const unsigned nb = (unsigned)((N + 255) / 256);
         sites_zero_kernel<<<(unsigned)((cells + 255) / 256), 256, 0, s>>>(ccnt, cells, mm);
-        sites_bbox_kernel<<<nb < 1024 ? nb : 1024, 256, 0, s>>>(sites, N, mm);
+        sites_bbox_kernel<<<nb < kBoxCtas ? nb : kBoxCtas, 256, 0, s>>>(sites, N, mm);
         // about 4 sites per grid cell: the warp search pays per ring (a
         // round of dependent loads) far more than per candidate (32 lanes)
         const int64_t cap = N / 4 > 4096 ? N / 4 : 4096;

@@ -171,6 +171,30 @@ __device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t d, uint32_t inv)
     return q;
 }
 
+// The box of a CTA's points into mm (smallest 0..2, largest 3..5): one atomic
+// a CTA and bound. With one a warp, the atomics on six words were most of a
+// bounding-box pass (200,000 points: 27 -> 4 to 6 us). Every thread calls it.
+__device__ __forceinline__ void cta_box_atomic(const int32_t lo[3], const int32_t hi[3], int32_t* mm)
+{
+    __shared__ int32_t s_box[6];
+    const unsigned full = 0xffffffffu;
+    if (threadIdx.x < 6) s_box[threadIdx.x] = threadIdx.x < 3 ? INT32_MAX : INT32_MIN;
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int32_t l = __reduce_min_sync(full, lo[a]), h = __reduce_max_sync(full, hi[a]);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&s_box[a], l);
+            atomicMax(&s_box[3 + a], h);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) atomicMin(&mm[threadIdx.x], s_box[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(&mm[threadIdx.x], s_box[threadIdx.x]);
+}
+// CTAs of 256 threads of such a pass (two an SM)
+constexpr unsigned kBoxCtas = 304;
+
 // Uniform grid over Gaussian bounding spheres, for the bake.
 struct GaussGrid {
     float origin[3];
