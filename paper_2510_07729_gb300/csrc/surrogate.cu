@@ -435,14 +435,7 @@ __global__ void __launch_bounds__(kNearThreads) surr_near_comp_kernel(const Near
     }
     __syncthreads();
     const int RR = k.R * k.R;
-    // a warp takes a tile of 8 x 4 texels where the map splits into them: its
-    // directions span a narrower cone than two rows of the map, so more
-    // Gaussians miss all of them (4,096 probes at R = 16: 524 -> 510 us)
-    const bool tiled = k.R % 8 == 0;
-    const int per_row = k.R / 8;
-    for (int t0 = tid; t0 < RR; t0 += kNearThreads) {
-        const int tile = t0 >> 5, l = t0 & 31;
-        const int t = tiled ? (tile / per_row * 4 + (l >> 3)) * k.R + tile % per_row * 8 + (l & 7) : t0;
+    for (int t = tid; t < RR; t += kNearThreads) {
         const float4 d4 = __ldg(k.tdirs + t);
         const float3 d = f3(d4.x, d4.y, d4.z);
         float T = 1.f, L0 = 0.f, L1 = 0.f, L2 = 0.f, W = 0.f, Dacc = 0.f;

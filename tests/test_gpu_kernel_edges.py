@@ -237,22 +237,3 @@ def test_bake_binning_paths_agree(sop, n, needles):
         assert bool(sop.device_status() & sop.DEVSTAT_GRID_COARSENED) == needles
         out.append((at.rgbo.cpu().numpy(), at.depth.cpu().numpy()))
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
-
-
-@pytest.mark.parametrize("R", [2, 7, 8, 24, 64])
-def test_surrogate_features_map_sizes(sop, orc, R):
-    """The near field's warps take tiles of 8 x 4 texels where the map's edge
-    is a multiple of 8 and texels in order elsewhere: every texel once, at
-    the bounds of the feature tests."""
-    from paper_2510_07729_gb300 import inputs as I
-    from tests.test_gpu_surrogate import R_NEAR, check_far, check_near, params
-    scene = I.surrogate_scene(1003, n_gauss=20000, n_probes=12)
-    g, pp = scene["gauss"], scene["probe_pos"]
-    net = sop.Surrogate(params(), r_near=R_NEAR)
-    gf, lst = net.features({k: cuda(v) for k, v in g.items()}, cuda(pp), R, with_list=True)
-    of, flags, olst, _, sens = orc.surr_features(g, pp, R, R_NEAR, far_sens=True)
-    gf = gf.cpu().numpy()
-    assert np.array_equal(lst.cpu().numpy(), olst)
-    ok = flags == 0
-    check_near(gf, of, ok, f"near field R={R}")
-    check_far(gf, of, sens, f"far field R={R}")
