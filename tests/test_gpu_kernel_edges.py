@@ -237,3 +237,4 @@ def test_bake_binning_paths_agree(sop, n, needles):
         assert bool(sop.device_status() & sop.DEVSTAT_GRID_COARSENED) == needles
         out.append((at.rgbo.cpu().numpy(), at.depth.cpu().numpy()))
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
