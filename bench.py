@@ -621,7 +621,11 @@ def compose_frame_variant(sop, dev, flush, steps, l2_gbs, hbm_gbs, peak_fp32, ba
         res[label] = {"frame_ms": round(ms, 4),
                       **{f"{q['name']}_ms": round(float(np.mean(tp[q["name"]])), 4) for q in st.parts},
                       "point_dirs_per_s": round(pd / (ms * 1e-3), 1),
-                      "roofline": {"kernel": "shade_kernel (the frame's two sop_query_shade calls)",
+                      "roofline": {"kernel": "shade_point_kernel + shadow_warp_kernel and their searches (the frame's "
+                                             "two sop_query_shade calls)",
+                                   "note": "l2 counts the texels of every point-direction; points on one normal "
+                                           "share a probe's directions in the SHADOW call, which moves fewer (frac "
+                                           "may exceed 1)",
                                    "bound": bound[1], "t_hbm_ms": round(t_hbm * 1e3, 4),
                                    "t_l2_ms": round(t_l2 * 1e3, 4), "t_alu_ms": round(t_alu * 1e3, 4),
                                    "frac": round(bound[0] * 1e3 / ms, 4), "l2_demand_bytes": int(dem),
