@@ -308,42 +308,70 @@ __device__ __forceinline__ void cell_range(const GaussGrid& G, const uint4 en, i
     }
 }
 
-// Gaussian i counted in its cells, or entered into them (after the scan of the
-// counts, which clears them).
-__device__ __forceinline__ void bin_count(int64_t i, const GRec* __restrict__ rec, const GaussGrid& G,
-                                          int32_t* __restrict__ cell_cnt)
+// f(cell, entry) for every cell of a warp's 32 Gaussians (thread's: i). The
+// pairs of Gaussian and cell are dealt to the lanes in order, 32 a round: a
+// lane that walked its own Gaussian's cells would wait for an atomic's answer
+// at each of them, with the warp as slow as its widest Gaussian (200,000
+// Gaussians, 10 cells each: counting 38 -> 20 us, filling 70 -> 39 us; bound
+// now by the atomics). Every lane calls it. WITH_ENTRY: f needs the entry
+// (else it is given zeros).
+template <bool WITH_ENTRY, class F>
+__device__ __forceinline__ void warp_cells(int64_t i, int64_t n, const GRec* __restrict__ rec, const GaussGrid& G, F f)
 {
-    const float4 r0 = rec[i].r0;
-    if (r0.w < 0.f) return;
-    int lo[3], hi[3];
-    cell_range(G, make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i), lo, hi);
-    for (int z = lo[2]; z <= hi[2]; ++z)
-        for (int y = lo[1]; y <= hi[1]; ++y)
-            for (int x = lo[0]; x <= hi[0]; ++x) atomicAdd(&cell_cnt[(z * G.dims[1] + y) * G.dims[0] + x], 1);
-}
-
-__device__ __forceinline__ void bin_fill(int64_t i, const GRec* __restrict__ rec, const GaussGrid& G,
-                                         const int32_t* __restrict__ cell_start, int32_t* __restrict__ cell_cnt,
-                                         uint4* __restrict__ ent)
-{
-    const float4 r0 = rec[i].r0;
-    if (r0.w < 0.f) return;
-    const uint4 en = make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i);
-    int lo[3], hi[3];
-    cell_range(G, en, lo, hi);
-    for (int z = lo[2]; z <= hi[2]; ++z)
-        for (int y = lo[1]; y <= hi[1]; ++y)
-            for (int x = lo[0]; x <= hi[0]; ++x) {
-                const int c = (z * G.dims[1] + y) * G.dims[0] + x;
-                ent[cell_start[c] + atomicAdd(&cell_cnt[c], 1)] = en;
-            }
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    uint4 en = make_uint4(0, 0, 0, 0);
+    int32_t first = 0;
+    uint32_t nx = 1, nxy = 1;
+    long long cnt = 0;
+    if (i < n) {
+        const float4 r0 = rec[i].r0;
+        if (!(r0.w < 0.f)) {
+            en = make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i);
+            int lo[3], hi[3];
+            cell_range(G, en, lo, hi);
+            first = (lo[2] * G.dims[1] + lo[1]) * G.dims[0] + lo[0];
+            nx = (uint32_t)(hi[0] - lo[0] + 1);
+            nxy = nx * (uint32_t)(hi[1] - lo[1] + 1);
+            cnt = (long long)nxy * (hi[2] - lo[2] + 1);
+        }
+    }
+    long long end = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long v = __shfl_up_sync(full, end, o);
+        if (lane >= o) end += v;
+    }
+    const long long begin = end - cnt, total = __shfl_sync(full, end, 31);
+    for (long long t0 = 0; t0 < total; t0 += 32) {
+        // the Gaussian of the round's pair `lane`: the first that ends after it
+        const long long left = end - t0;
+        const int rel = left < 0 ? 0 : (left > 32 ? 32 : (int)left);
+        int o = 0;
+#pragma unroll
+        for (int step = 16; step; step >>= 1)
+            if (__shfl_sync(full, rel, o + step - 1) <= lane) o += step;
+        const uint32_t j = (uint32_t)lane - __shfl_sync(full, (uint32_t)(begin - t0), o);
+        const int32_t c0 = __shfl_sync(full, first, o);
+        const uint32_t w = __shfl_sync(full, nx, o), wh = __shfl_sync(full, nxy, o);
+        const uint32_t z = j / wh, r = j - z * wh, y = r / w, x = r - y * w;
+        uint4 e = make_uint4(0, 0, 0, 0);
+        if (WITH_ENTRY) {
+            e.x = __shfl_sync(full, en.x, o);
+            e.y = __shfl_sync(full, en.y, o);
+            e.z = __shfl_sync(full, en.z, o);
+            e.w = __shfl_sync(full, en.w, o);
+        }
+        if (t0 + lane < total) f(c0 + ((int32_t)z * G.dims[1] + (int32_t)y) * G.dims[0] + (int32_t)x, e);
+    }
 }
 
 __global__ void bin_count_kernel(int64_t N, const GRec* __restrict__ rec, const GaussGrid* __restrict__ gridp,
                                  int32_t* __restrict__ cell_cnt)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) bin_count(i, rec, *gridp, cell_cnt);
+    const GaussGrid G = *gridp;
+    warp_cells<false>(i, N, rec, G, [&](int c, const uint4&) { atomicAdd(cell_cnt + c, 1); });
 }
 
 // After the scan of a binning attempt's counts: whether the cell lists fit
@@ -367,7 +395,11 @@ __global__ void bin_fill_kernel(int64_t N, const GRec* __restrict__ rec, const G
                                 uint4* __restrict__ ent)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N && gridp->fits) bin_fill(i, rec, *gridp, cell_start, cell_cnt, ent);
+    const GaussGrid G = *gridp;
+    if (!G.fits) return;
+    warp_cells<true>(i, N, rec, G, [&](int c, const uint4& en) {
+        ent[__ldg(cell_start + c) + atomicAdd(cell_cnt + c, 1)] = en;
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -400,7 +432,9 @@ struct BinK {
 
 constexpr int kBinSmemCells = 8192;  // cells counted in shared memory
 
-// f(cell, entry) for the cells of the CTA's Gaussians
+// f(cell, entry) for the cells of the CTA's Gaussians; a thread a Gaussian,
+// whose atomics are in shared memory here (dealt to the lanes: a bake of 2,000
+// Gaussians 76 -> 78 us)
 template <class F>
 __device__ __forceinline__ void bin_visit(int64_t n, const GRec* __restrict__ rec, const GaussGrid& G, F f)
 {
