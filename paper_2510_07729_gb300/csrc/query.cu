@@ -304,7 +304,8 @@ __device__ __forceinline__ uint64_t unsearched_bound2(const ProbeGrid& G, const 
 // instructions instead of 10. A cell whose nearest point lies beyond the K-th
 // kept key is not read. 2,051,693 pixels of a ground frame, 4,096 probes,
 // K = 8: 497 -> 405 us (5,290 instructions a warp); an object view of 418,111:
-// 178 -> 155 us.
+// 178 -> 155 us. Nine CTAs an SM (56 registers, 24 bytes spilled) instead of
+// eight: the frame's whole call 694 -> 678 us, ten (48, 88 bytes): 680.
 // ---------------------------------------------------------------------------
 // squared distance along one axis from q to the cell interval [lo, lo + cs)
 __device__ __forceinline__ uint64_t axis_gap2(int32_t q, int64_t lo, int32_t cs)
@@ -402,7 +403,7 @@ __device__ __forceinline__ void knn_search(const ProbeGrid& G, const int32_t q[3
 }
 
 template <int KMAX>
-__global__ void __launch_bounds__(128, KMAX <= 8 ? 8 : 1) knn_kernel(const float* __restrict__ x, const float* __restrict__ nrm, int64_t M,
+__global__ void __launch_bounds__(128, KMAX <= 8 ? 9 : 1) knn_kernel(const float* __restrict__ x, const float* __restrict__ nrm, int64_t M,
                                                    int32_t K, int32_t id_bits, uint64_t snap_key, uint64_t r2_key,
                                                    const ProbeGrid* __restrict__ gridp,
                                                    const int32_t* __restrict__ cell_start,
@@ -1439,9 +1440,10 @@ __global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
 // Query + shade, SHADE mode, one warp per point (point_blend.cuh): lanes
 // share the directions, 32 a round. NR: rounds whose footprints stay in
 // registers between the marking and the shading (S <= 32 NR), or 0: any S,
-// computed twice. Bound: L2 for the blended texels (20 KB a point at R = 16,
-// K = 8), then L1 gathers of the environment. 418,111 points, K = 8, S = 128:
-// 1,717 -> 1,400 us against shade_kernel.
+// computed twice. Bound: L1 and shared memory (92% of their throughput): the
+// blended texels (20 KB a point at R = 16, K = 8), four of them a direction
+// from shared memory, the environment's gathers. 418,111 points, K = 8,
+// S = 128: 1,717 -> 1,400 us against shade_kernel.
 // ---------------------------------------------------------------------------
 template <int DT, int KMAX, int NR>
 __global__ void __launch_bounds__(kPointWarps * 32, 4) shade_point_kernel(const ShadeK a)
