@@ -628,7 +628,6 @@ __global__ void __launch_bounds__(kAdjPts * 32, 2) adjoint_tile_kernel(const Adj
             const float iden = __fdividef(1.f, NdotH * NdotH * a2 + sin2), igl = __fdividef(1.f, NdotL * (1.f - kk) + kk);
             const float ip2 = kInvPi * iden * iden, D = a2 * ip2, Gc = igl * G1Vn, spec_t = D * Gc;
             const float x1 = 1.f - VdotH, x2 = x1 * x1, fc = x2 * x2 * x1;
-            const float ip3 = ip2 * iden;
             const float dspec_dr = (1.f - 2.f * a2 * NdotH * NdotH * iden) * ip2 * r3 * Gc +
                                    D * cr0 * igl * (cr1 - (1.f - NdotL) * igl * G1V);
             float gLd[3], SF = 0.f, SV = 0.f;
@@ -648,8 +647,10 @@ __global__ void __launch_bounds__(kAdjPts * 32, 2) adjoint_tile_kernel(const Adj
                 gO -= gLin[c] * Ld;
             }
             gr += SF * dspec_dr;
-            // dL/d(n.h), dL/d|n x h|^2, dL/d(v.h), dL/d(n.v)
-            const float GN = SF * Gc * (-4.f * a2 * a2 * NdotH * ip3), GS = SF * Gc * (-2.f * a2 * ip3);
+            // dL/d(n.h), dL/d|n x h|^2, dL/d(v.h), dL/d(n.v). (-2 a2 / (pi den^3)
+            // as -2 D / den: den is r^4 at the mirror direction, whose inverse
+            // cube alone leaves float32 below r = 5.6e-4)
+            const float GS = SF * Gc * (-2.f * (D * iden)), GN = 2.f * a2 * NdotH * GS;
             const float GVH = SV * spec_t * (-5.f * x2 * x2), GNV = SF * D * igl * cnv;
             // ---- scatter: environment -------------------------------------------
 #pragma unroll
@@ -689,16 +690,15 @@ __global__ void __launch_bounds__(kAdjPts * 32, 2) adjoint_tile_kernel(const Adj
             }
             // BRDF geometry through h, and directly through n
             const float hh[3] = {h.x, h.y, h.z}, nn[3] = {n.x, n.y, n.z}, vv[3] = {wo.x, wo.y, wo.z};
-            const float ln = GN - 2.f * GS * NdotH;
             float gh[3];
 #pragma unroll
-            for (int j = 0; j < 3; ++j) gh[j] = ln * nn[j] + 2.f * GS * hh[j] + GVH * vv[j];
+            for (int j = 0; j < 3; ++j) gh[j] = GN * nn[j] + 2.f * GS * (hh[j] - NdotH * nn[j]) + GVH * vv[j];
             const float hg = hh[0] * gh[0] + hh[1] * gh[1] + hh[2] * gh[2];
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 gw[j] += (gh[j] - hg * hh[j]) * ihl;
                 // w = l.x t(n) + l.y b(n) + l.z n
-                gn[j] += l.z * gw[j] + (ln * hh[j] + 2.f * GS * nn[j] + GNV * vv[j]);
+                gn[j] += l.z * gw[j] + (GN * hh[j] + 2.f * GS * (nn[j] - NdotH * hh[j]) + GNV * vv[j]);
                 gt[j] += l.x * gw[j];
                 gb[j] += l.y * gw[j];
             }
