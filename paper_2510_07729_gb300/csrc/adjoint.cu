@@ -619,16 +619,15 @@ __global__ void __launch_bounds__(kAdjPts * 32, 2) adjoint_tile_kernel(const Adj
             // ---- BRDF -----------------------------------------------------------
             const float3 hv = w + wo;
             const float hl2 = dot3(hv, hv);
-            float ihl = hl2 > 1e-30f ? rsqrtf(hl2) : 0.f;
-            ihl *= fmaf(-0.5f * hl2 * ihl, ihl, 1.5f);  // (one Newton step: a fraction of an ulp)
+            const float ihl = hl2 > 1e-30f ? 1.f / sqrtf(hl2) : 0.f;
             const float3 h = hl2 > 1e-30f ? ihl * hv : n;
             const float NdotH = dot3(n, h), VdotH = dot3(wo, h);
             const float3 cr = cross3(n, h);
             const float sin2 = dot3(cr, cr);
-            const float iden = __fdividef(1.f, NdotH * NdotH * a2 + sin2), igl = __fdividef(1.f, NdotL * (1.f - kk) + kk);
+            const float den = NdotH * NdotH * a2 + sin2, iden = 1.f / den, igl = 1.f / (NdotL * (1.f - kk) + kk);
             const float ip2 = kInvPi * iden * iden, D = a2 * ip2, Gc = igl * G1Vn, spec_t = D * Gc;
             const float x1 = 1.f - VdotH, x2 = x1 * x1, fc = x2 * x2 * x1;
-            const float dspec_dr = (1.f - 2.f * a2 * NdotH * NdotH * iden) * ip2 * r3 * Gc +
+            const float dspec_dr = (den - 2.f * a2 * NdotH * NdotH) * iden * ip2 * r3 * Gc +
                                    D * cr0 * igl * (cr1 - (1.f - NdotL) * igl * G1V);
             float gLd[3], SF = 0.f, SV = 0.f;
             const float s1 = spec_t * (1.f - fc);
@@ -667,7 +666,7 @@ __global__ void __launch_bounds__(kAdjPts * 32, 2) adjoint_tile_kernel(const Adj
             const float gu = ((1.f - fv) * dotg(d10) + fv * dotg(d11)) * Rf;
             const float gv = ((1.f - fu) * dotg(e01) + fu * dotg(e11)) * Rf;
             const float ax_ = fabsf(w.x), ay_ = fabsf(w.y), az_ = fabsf(w.z);
-            const float l1 = ax_ + ay_ + az_, il2 = __fdividef(1.f, l1 * l1);
+            const float l1 = ax_ + ay_ + az_, il2 = 1.f / (l1 * l1);
             const float sx = w.x >= 0.f ? 1.f : -1.f, sy = w.y >= 0.f ? 1.f : -1.f, sz = w.z >= 0.f ? 1.f : -1.f;
             const float fold = w.z < 0.f ? -sx * sy : 0.f;
             const float px = 0.5f * il2 * (w.z < 0.f ? fold * gv : gu), py = 0.5f * il2 * (w.z < 0.f ? fold * gu : gv);
