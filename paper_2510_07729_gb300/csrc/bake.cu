@@ -52,8 +52,14 @@ static int64_t cells_cap_for(int64_t N, float density)
     return c < 4096 ? 4096 : (c > (1 << 23) ? (1 << 23) : c);
 }
 
-// binning attempts of launch_bake_bin
+// Binning attempts, decided on the device (no host read-back): the requested
+// grid; if its cell lists overflow the workspace, a grid with 1/16 of the
+// cells; then one of at most 2 cells, whose lists (at most 2 entries per
+// Gaussian) always fit, since the workspace holds at least 24 per Gaussian.
 constexpr int kBinAttempts = 3;
+// words of the box's 16 that bin_coarse_kernel uses: CTAs done, and the two
+// counts of the last attempt's cells
+constexpr int kBinTicket = 8, kBinTwo = 9;
 
 BakeLayout bake_layout(int64_t N, int64_t entries_cap, float density)
 {
@@ -254,6 +260,7 @@ __global__ void __launch_bounds__(1024) grid_setup_kernel(const int32_t* __restr
     cta_box(lo, hi, s_box, box);
     if (threadIdx.x == 0) {
         for (int a = 0; a < 6; ++a) bbox[a] = box[a];
+        for (int a = kBinTicket; a < kBinTwo + 2; ++a) bbox[a] = 0;
         *grid = grid_geometry(box, cells_cap, 0);
     }
 }
@@ -402,20 +409,6 @@ __global__ void bin_fill_kernel(int64_t N, const GRec* __restrict__ rec, const G
     });
 }
 
-// ---------------------------------------------------------------------------
-// Binning by one CTA. For small sets (kBinOneCta) it does all of it, records
-// included, with the cells counted in shared memory, where the general path's
-// seven launches are most of the time (2,000 Gaussians: a bake of 64 probes
-// 122 us with 22 launches, 77 us with 4; 24 us of it here, a third waiting
-// for the parameters); for larger ones it is the later attempts' launch,
-// which returns at once when the first grid fitted.
-// Attempts (decided on the device, no host read-back): the requested grid; if
-// its cell lists overflow the workspace, a grid with 1/16 of the cells; then
-// one of at most 2 cells, whose lists (at most 2 entries per Gaussian) always
-// fit, since the workspace holds at least 24 per Gaussian.
-// ---------------------------------------------------------------------------
-constexpr int64_t kBinOneCta = 4096;
-
 struct BinK {
     sop_gaussians g;
     float alpha_min;
@@ -426,109 +419,209 @@ struct BinK {
     int32_t *bbox, *cell_start, *cell_cnt;
     uint4* ent;
     unsigned int* status;
-    int32_t first;  // 0: every attempt; 1: those after the first
-    int32_t prep;   // compute the records and the box too
 };
 
-constexpr int kBinSmemCells = 8192;  // cells counted in shared memory
-
-// f(cell, entry) for the cells of the CTA's Gaussians; a thread a Gaussian,
-// whose atomics are in shared memory here (dealt to the lanes: a bake of 2,000
-// Gaussians 76 -> 78 us)
-template <class F>
-__device__ __forceinline__ void bin_visit(int64_t n, const GRec* __restrict__ rec, const GaussGrid& G, F f)
+// The cells of one Gaussian: first + (z dims_1 + y) dims_0 + x below (nx, ny, nz).
+struct CellBox {
+    int32_t first, nx, ny, nz;
+};
+__device__ __forceinline__ CellBox cell_box(const GaussGrid& G, const uint4 en)
 {
-    for (int64_t i = threadIdx.x; i < n; i += 1024) {
-        const float4 r0 = rec[i].r0;
-        if (r0.w < 0.f) continue;
-        const uint4 en = make_entry(G, f3(r0.x, r0.y, r0.z), rec[i].r4, (int32_t)i);
-        int lo[3], hi[3];
-        cell_range(G, en, lo, hi);
-        for (int z = lo[2]; z <= hi[2]; ++z)
-            for (int y = lo[1]; y <= hi[1]; ++y)
-                for (int x = lo[0]; x <= hi[0]; ++x) f((z * G.dims[1] + y) * G.dims[0] + x, en);
-    }
+    int lo[3], hi[3];
+    cell_range(G, en, lo, hi);
+    return {(lo[2] * G.dims[1] + lo[1]) * G.dims[0] + lo[0], hi[0] - lo[0] + 1, hi[1] - lo[1] + 1, hi[2] - lo[2] + 1};
 }
+template <class F>
+__device__ __forceinline__ void each_cell(const int dx, const int dxy, const CellBox& b, F f)
+{
+    for (int z = 0; z < b.nz; ++z)
+        for (int y = 0; y < b.ny; ++y)
+            for (int x = 0, c = b.first + z * dxy + y * dx; x < b.nx; ++x, ++c) f(c);
+}
+
+// ---------------------------------------------------------------------------
+// Binning of a small set by one CTA, records included, with the cells counted
+// in shared memory, where the general path's seven launches are most of the
+// time (2,000 Gaussians: a bake of 64 probes 122 us with 22 launches, 77 us
+// with 4; 24 us of it here, a third waiting for the parameters). The lists'
+// length is the sum of the boxes' volumes, so an attempt that does not fit is
+// left before a cell of it is counted: what one CTA counts and fills is
+// bounded by kBinOneEntries (4,096 Gaussians over all cells: 515 us with every
+// attempt counted, 252 us now).
+// ---------------------------------------------------------------------------
+constexpr int64_t kBinOneCta = 4096;
+constexpr int kBinOnePer = (int)(kBinOneCta / 1024);  // Gaussians a thread
+constexpr int kBinSmemCells = 8192;                   // cells counted in shared memory
+// entry capacity of the smallest workspace of kBinOneCta Gaussians; with more
+// (a caller's extra bytes) the lists may be longer than is good for one CTA
+constexpr int64_t kBinOneEntries = 24 * kBinOneCta + 65536 + 4096;
 
 __global__ void __launch_bounds__(1024) bin_one_kernel(const BinK k)
 {
     __shared__ int32_t s_box[6][32];
     __shared__ long long s_w[kScanThreads / 32];
     __shared__ GaussGrid G;
-    __shared__ long long s_tot;
     __shared__ int32_t s_cnt[kBinSmemCells];
     const int tid = threadIdx.x;
-    if (k.first > 0 && k.grid->fits) return;
-    if (k.prep) {
-        float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-        for (int64_t i = tid; i < k.g.n; i += 1024) gauss_record(k.g, i, k.alpha_min, k.rec, k.status, lo, hi);
-        int32_t box[6];
-        cta_box(lo, hi, s_box, box);
-        if (tid == 0)
-            for (int a = 0; a < 6; ++a) k.bbox[a] = box[a];
-    }
+    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
+    for (int64_t i = tid; i < k.g.n; i += 1024) gauss_record(k.g, i, k.alpha_min, k.rec, k.status, lo, hi);
+    int32_t box[6];
+    cta_box(lo, hi, s_box, box);
     __syncthreads();
-    bool in_smem = false;
-    for (int level = k.first; level < kBinAttempts; ++level) {
-        if (tid == 0) {
-            int32_t box[6];
-            for (int a = 0; a < 6; ++a) box[a] = k.bbox[a];
-            G = grid_geometry(box, k.caps[level], level);
-            s_tot = 0;
-        }
+    const auto entry = [&](int64_t i) {
+        const float4 r0 = k.rec[i].r0;
+        return make_entry(G, f3(r0.x, r0.y, r0.z), k.rec[i].r4, (int32_t)i);
+    };
+    CellBox b[kBinOnePer];
+    for (int level = 0; level < kBinAttempts; ++level) {
+        if (tid == 0) G = grid_geometry(box, k.caps[level], level);
         __syncthreads();
-        const int nc = G.ncells;
-        in_smem = nc <= kBinSmemCells;
-        int32_t* cnt = in_smem ? s_cnt : k.cell_cnt;
-        for (int c = tid; c < nc; c += 1024) cnt[c] = 0;
-        __syncthreads();
-        bin_visit(k.g.n, k.rec, G, [&](int c, const uint4&) { atomicAdd(cnt + c, 1); });
-        __syncthreads();
-        // exclusive scan of the counts, a tile of them at a time; in shared
-        // memory they become the fill's cursors, else they are cleared
-        for (int c0 = 0; c0 < nc; c0 += kScanTile) {
-            int32_t v[kScanPer];
-            long long sum = 0, tot;
+        long long sum = 0, tot;
 #pragma unroll
-            for (int e = 0; e < kScanPer; ++e) {
-                const int c = c0 + tid * kScanPer + e;
-                v[e] = c >= nc ? 0 : (in_smem ? s_cnt[c] : __ldcg(k.cell_cnt + c));  // (counted by atomics in L2)
-                sum += v[e];
-            }
-            long long run = scan_block_inclusive(sum, s_w, &tot) - sum + s_tot;
-#pragma unroll
-            for (int e = 0; e < kScanPer; ++e) {
-                const int c = c0 + tid * kScanPer + e;
-                if (c < nc) {
-                    const int32_t at = (int32_t)(run < INT32_MAX ? run : INT32_MAX);
-                    k.cell_start[c] = at;
-                    cnt[c] = in_smem ? at : 0;
-                }
-                run += v[e];
-            }
-            __syncthreads();
-            if (tid == 0) s_tot += tot;
-            __syncthreads();
+        for (int j = 0; j < kBinOnePer; ++j) {
+            const int64_t i = tid + 1024 * j;
+            b[j] = {0, 0, 0, 0};
+            if (i < k.g.n && !(k.rec[i].r0.w < 0.f)) b[j] = cell_box(G, entry(i));
+            sum += (long long)b[j].nx * b[j].ny * b[j].nz;
         }
+        scan_block_inclusive(sum, s_w, &tot);
         if (tid == 0) {
-            k.cell_start[nc] = (int32_t)(s_tot < INT32_MAX ? s_tot : INT32_MAX);
-            BinScanFinal{&G, k.entries_cap, k.status}(s_tot);
+            BinScanFinal{&G, k.entries_cap, k.status}(tot);
             *k.grid = G;
         }
         __syncthreads();
         if (G.fits) break;
     }
     if (!G.fits) return;
-    if (!k.ent) {  // a launch of its own fills, with cleared counters
-        if (in_smem)
-            for (int c = tid; c < G.ncells; c += 1024) k.cell_cnt[c] = 0;
-    } else if (in_smem) {
-        bin_visit(k.g.n, k.rec, G, [&](int c, const uint4& en) { k.ent[atomicAdd(s_cnt + c, 1)] = en; });
-    } else {
-        bin_visit(k.g.n, k.rec, G, [&](int c, const uint4& en) {
-            k.ent[k.cell_start[c] + atomicAdd(k.cell_cnt + c, 1)] = en;
-        });
+    const int nc = G.ncells, dx = G.dims[0], dxy = dx * G.dims[1];
+    for (int c = tid; c < nc; c += 1024) s_cnt[c] = 0;
+    __syncthreads();
+    // a thread a Gaussian, whose atomics are in shared memory here (pairs
+    // dealt to the lanes: a bake of 2,000 Gaussians 76 -> 78 us)
+#pragma unroll
+    for (int j = 0; j < kBinOnePer; ++j) each_cell(dx, dxy, b[j], [&](int c) { atomicAdd(s_cnt + c, 1); });
+    __syncthreads();
+    // exclusive scan of the counts, a tile of them at a time; they become the
+    // fill's cursors
+    long long before = 0;
+    for (int c0 = 0; c0 < nc; c0 += kScanTile) {
+        int32_t v[kScanPer];
+        long long sum = 0, tot;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            const int c = c0 + tid * kScanPer + e;
+            v[e] = c < nc ? s_cnt[c] : 0;
+            sum += v[e];
+        }
+        long long run = scan_block_inclusive(sum, s_w, &tot) - sum + before;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            const int c = c0 + tid * kScanPer + e;
+            if (c < nc) k.cell_start[c] = s_cnt[c] = (int32_t)run;  // (the lists fit 32 bits)
+            run += v[e];
+        }
+        before += tot;
+        __syncthreads();
     }
+    if (tid == 0) k.cell_start[nc] = (int32_t)before;
+#pragma unroll
+    for (int j = 0; j < kBinOnePer; ++j)
+        if (b[j].nx > 0) {
+            const uint4 en = entry(tid + 1024 * j);
+            each_cell(dx, dxy, b[j], [&](int c) { k.ent[atomicAdd(s_cnt + c, 1)] = en; });
+        }
+}
+
+// ---------------------------------------------------------------------------
+// The attempts after the first of a larger set, in one launch that returns at
+// once when the first grid fitted: every CTA counts its Gaussians in the grid
+// with 1/16 of the cells and in the one of at most two, and the last CTA to
+// finish (a ticket; nothing waits) scans the first one's counts, a tile at a
+// time, and takes the second where they do not fit either. The fill follows.
+// 20,000 / 200,000 / 1,000,000 Gaussians whose lists overflow, binning in all:
+// 115 / 235 / 837 us; 286 / 2,560 / 15,170 with one CTA for these attempts, 199
+// / 442 / 1,300 with five launches for each.
+// ---------------------------------------------------------------------------
+constexpr unsigned kCoarseCtas = 304;  // of 1,024 threads (two an SM)
+
+__global__ void __launch_bounds__(1024) bin_coarse_kernel(const BinK k)
+{
+    __shared__ GaussGrid G1, G2;
+    __shared__ long long s_w[kScanThreads / 32];
+    __shared__ int32_t s_two[2];
+    __shared__ bool s_last;
+    if (k.grid->fits) return;
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) {
+        int32_t box[6];
+        for (int a = 0; a < 6; ++a) box[a] = k.bbox[a];
+        G1 = grid_geometry(box, k.caps[1], 1);
+        G2 = grid_geometry(box, k.caps[2], 2);
+        s_two[0] = s_two[1] = 0;
+    }
+    __syncthreads();
+    for (int64_t i0 = (int64_t)blockIdx.x * 1024; i0 < k.g.n; i0 += (int64_t)gridDim.x * 1024) {
+        const int64_t i = i0 + tid;
+        warp_cells<false>(i, k.g.n, k.rec, G1, [&](int c, const uint4&) { atomicAdd(k.cell_cnt + c, 1); });
+        CellBox b = {2, 1, 1, 1};
+        if (i < k.g.n) {
+            const float4 r0 = k.rec[i].r0;
+            if (!(r0.w < 0.f)) b = cell_box(G2, make_entry(G2, f3(r0.x, r0.y, r0.z), k.rec[i].r4, (int32_t)i));
+        }
+        // (at most two cells: a box takes the first, the second or both)
+        const unsigned m0 = __ballot_sync(full, b.first == 0);
+        const unsigned m1 = __ballot_sync(full, b.first == 1 || (b.first == 0 && b.nx * b.ny * b.nz == 2));
+        if (lane == 0) {
+            if (m0) atomicAdd(&s_two[0], __popc(m0));
+            if (m1) atomicAdd(&s_two[1], __popc(m1));
+        }
+    }
+    __syncthreads();
+    if (tid < 2 && s_two[tid]) atomicAdd(k.bbox + kBinTwo + tid, s_two[tid]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(k.bbox + kBinTicket, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    long long before = 0;
+    const int nc = G1.ncells;
+    for (int c0 = 0; c0 < nc; c0 += kScanTile) {
+        int32_t v[kScanPer];
+        long long sum = 0, tot;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            const int c = c0 + tid * kScanPer + e;
+            v[e] = c < nc ? __ldcg(k.cell_cnt + c) : 0;  // (counted by atomics in L2)
+            sum += v[e];
+        }
+        long long run = scan_block_inclusive(sum, s_w, &tot) - sum + before;
+#pragma unroll
+        for (int e = 0; e < kScanPer; ++e) {
+            const int c = c0 + tid * kScanPer + e;
+            if (c < nc) {
+                k.cell_start[c] = (int32_t)(run < INT32_MAX ? run : INT32_MAX);
+                k.cell_cnt[c] = 0;
+            }
+            run += v[e];
+        }
+        before += tot;
+        __syncthreads();
+    }
+    if (tid != 0) return;
+    BinScanFinal{&G1, k.entries_cap, k.status}(before);
+    if (G1.fits) {
+        k.cell_start[nc] = (int32_t)before;
+        *k.grid = G1;
+        return;
+    }
+    const int32_t n0 = __ldcg(k.bbox + kBinTwo), n1 = __ldcg(k.bbox + kBinTwo + 1);
+    k.cell_start[0] = 0;
+    k.cell_start[1] = n0;
+    if (G2.ncells > 1) k.cell_start[2] = n0 + n1;
+    BinScanFinal{&G2, k.entries_cap, k.status}((long long)n0 + n1);
+    *k.grid = G2;
 }
 
 // Start of a bake's trace: the counters cleared, and the texel-centre
@@ -1241,14 +1334,12 @@ static BinK bin_args(const sop_gaussians& g, float alpha_min, const BakeLayout& 
     k.cell_cnt = reinterpret_cast<int32_t*>(ws + L.cell_cnt);
     k.ent = reinterpret_cast<uint4*>(ws + L.ent);
     k.status = status_word();
-    k.first = 0;
-    k.prep = 1;
     return k;
 }
 
 cudaError_t launch_bake_bin(const sop_gaussians& g, float alpha_min, const BakeLayout& L, char* ws, cudaStream_t s)
 {
-    if (g.n <= kBinOneCta) {
+    if (g.n <= kBinOneCta && L.cells_cap <= kBinSmemCells && L.entries_cap <= kBinOneEntries) {
         bin_one_kernel<<<1, 1024, 0, s>>>(bin_args(g, alpha_min, L, ws));
         return cudaGetLastError();
     }
@@ -1256,16 +1347,16 @@ cudaError_t launch_bake_bin(const sop_gaussians& g, float alpha_min, const BakeL
     return e != cudaSuccess ? e : launch_bake_grid(g, L, ws, s);
 }
 
-// CTAs of gauss_prep_kernel; their boxes wait in the entries' space
-static unsigned prep_parts(int64_t n) { return (unsigned)((n + 255) / 256); }
+// CTAs of gauss_prep_kernel (one clears the counters of an empty set); their
+// boxes wait in the entries' space
+static unsigned prep_parts(int64_t n) { return n > 0 ? (unsigned)((n + 255) / 256) : 1u; }
 
 cudaError_t launch_bake_prep(const sop_gaussians& g, float alpha_min, const BakeLayout& L, char* ws, cudaStream_t s)
 {
-    if (g.n > 0)
-        gauss_prep_kernel<<<prep_parts(g.n), 256, 0, s>>>(g, alpha_min, reinterpret_cast<GRec*>(ws + L.rec),
-                                                          reinterpret_cast<int32_t*>(ws + L.ent),
-                                                          reinterpret_cast<int32_t*>(ws + L.cell_cnt), L.cells_cap,
-                                                          status_word());
+    gauss_prep_kernel<<<prep_parts(g.n), 256, 0, s>>>(g, alpha_min, reinterpret_cast<GRec*>(ws + L.rec),
+                                                      reinterpret_cast<int32_t*>(ws + L.ent),
+                                                      reinterpret_cast<int32_t*>(ws + L.cell_cnt), L.cells_cap,
+                                                      status_word());
     return cudaGetLastError();
 }
 
@@ -1282,12 +1373,9 @@ cudaError_t launch_bake_grid(const sop_gaussians& g, const BakeLayout& L, char* 
     sa.start = k.cell_start;
     sa.scratch = reinterpret_cast<long long*>(ws + L.scan);
     launch_scan(sa, k.caps[0], BinScanFinal{k.grid, L.entries_cap, k.status}, s);
-    uint4* ent = k.ent;
-    k.first = 1;
-    k.prep = 0;
-    k.ent = nullptr;
-    bin_one_kernel<<<1, 1024, 0, s>>>(k);
-    if (g.n > 0) bin_fill_kernel<<<nb, 256, 0, s>>>(g.n, k.rec, k.grid, k.cell_start, k.cell_cnt, ent);
+    const int64_t nc = (g.n + 1023) / 1024;
+    bin_coarse_kernel<<<(unsigned)(nc < 1 ? 1 : (nc < kCoarseCtas ? nc : kCoarseCtas)), 1024, 0, s>>>(k);
+    if (g.n > 0) bin_fill_kernel<<<nb, 256, 0, s>>>(g.n, k.rec, k.grid, k.cell_start, k.cell_cnt, k.ent);
     return cudaGetLastError();
 }
 

@@ -4,6 +4,8 @@ import numpy as np
 import pytest
 import torch
 
+from tests.tolerance import assert_close
+
 pytestmark = pytest.mark.gpu
 F = np.float32
 
@@ -50,3 +52,52 @@ def test_adjoint_at_the_mirror_direction(sop, orc, rough):
     for got, ref in ((g["env"], w["env"]), (g["maps"][..., :3], w["maps_rgb"]), (g["maps"][..., 3], w["maps_occ"])):
         d = np.abs(got.cpu().numpy() - ref)
         assert np.all(d <= 1e-4 * np.abs(ref) + 2e-5 * np.abs(ref).max() + 1e-12)
+
+
+def _rods(n, length, width, diagonal, seed):
+    """Gaussians of one long and two short axes; along the space diagonals their
+    boxes are cubes of nearly the rods' length."""
+    rng = np.random.default_rng(seed)
+    u = rng.standard_normal((n, 3))
+    if diagonal:
+        u = np.sign(u) + 0.05 * rng.standard_normal((n, 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True).clip(1e-9)
+    q = np.stack([1 + u[:, 0], 0 * u[:, 0], -u[:, 2], u[:, 1]], axis=1)  # x to u
+    g = dict(mean=rng.uniform(-1, 1, (n, 3)), scale=np.tile([length, width, width], (n, 1)),
+             quat=q / np.linalg.norm(q, axis=1, keepdims=True).clip(1e-9), opacity=rng.uniform(0.05, 0.3, n),
+             rgb=rng.uniform(0, 1, (n, 3)))
+    return {k: v.astype(F) for k, v in g.items()}
+
+
+@pytest.mark.parametrize("n,length,width,two,extra", [
+    (0, 0.1, 0.01, False, 1 << 22),             # nothing to bin, in a workspace with room
+    (4096, 0.4, 0.01, False, 0), (4096, 3.0, 0.02, True, 0),         # one CTA
+    (4096, 0.4, 0.01, False, 1 << 24),                               # room for the first grid's lists: many CTAs
+    (5000, 3.0, 0.02, True, 0), (30_000, 0.15, 0.004, False, 0),     # many CTAs
+    (190_000, 0.05, 0.004, False, 0), (190_000, 0.15, 0.002, True, 0),  # more than 8,192 coarse cells
+])
+def test_coarsened_bakes(sop, orc, n, length, width, two, extra):
+    """Sets whose cell lists overflow the workspace, binned by one CTA and by
+    many into the grid of 1/16 of the cells and into the one of two (`two`:
+    diagonal rods, which overflow the former too): the traced maps against the
+    oracle (the bakes' bound: 1e-5 and the rounding of the texel directions;
+    occlusion alone where two hits are within rounding of each other)."""
+    g, R = _rods(n, length, width, two, n), 4
+    far = 1.5 + (3.6 * length if n < 10_000 else 0.6)  # outside every box: no hits with one entry point
+    out = np.concatenate([np.eye(3), -np.eye(3)]) * far + 0.1
+    pp = (out if two else np.array([[0.1, 0.2, -0.1], [0.4, -0.3, 0.2]])).astype(F)
+    ws = sop.BakeWorkspace(n, "cuda", extra_bytes=extra)
+    at = sop.make_atlas(cuda(pp), R)
+    sop.device_status()
+    sop.bake({k: cuda(v) for k, v in g.items()}, at, t_stop=0.0, workspace=ws)
+    assert bool(sop.device_status() & sop.DEVSTAT_GRID_COARSENED) == (n > 0 and extra == 0)
+    rgb, occ, dep = (t.cpu().numpy() for t in at.interior())
+    if n == 0:
+        assert not occ.any() and not rgb.any()
+        return
+    o_rgb, o_occ, o_dep, fl, sens = orc.bake(g, pp, R, t_stop=0.0, with_sens=True)
+    decided = (fl & (orc.FLAG_ALPHA_MIN | orc.FLAG_TNEAR | orc.FLAG_TSTOP)) == 0
+    assert (decided & (o_occ > 0.1)).sum() >= 6  # enough rays through many Gaussians
+    assert_close(occ[decided], o_occ[decided], what="O", absolute=sens[..., 3][decided])
+    ok = decided & ((fl & orc.FLAG_ORDER) == 0)
+    assert_close(rgb[ok], o_rgb[ok], what="L_in", absolute=sens[..., :3][ok])
