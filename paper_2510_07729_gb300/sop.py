@@ -7,8 +7,10 @@ or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
+import collections
 import ctypes as C
 import os
+import threading
 from dataclasses import dataclass, field
 
 import torch
@@ -200,6 +202,37 @@ def _stream():
 def _ws(nbytes, device):
     # 256-byte aligned scratch from torch's caching allocator
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
+
+
+def _capturing():
+    return torch.cuda.is_current_stream_capturing()
+
+
+class _StreamScratch:
+    """Scratch kept between calls, one buffer a device and stream, since calls
+    on two streams run side by side. At most `most` streams' buffers are kept
+    (the least recently used one goes); a buffer is allocated on the stream that
+    uses it, so the allocator gives a dropped one only to later work of that
+    stream. Hold `lock` from get() until the call that uses the buffer is
+    enqueued: another thread's call on the same stream then comes after it. A
+    call under capture gets a buffer of its graph's."""
+
+    def __init__(self, most=4):
+        self.lock = threading.Lock()
+        self._most = most
+        self._kept = collections.OrderedDict()
+
+    def get(self, device, key, make):
+        if _capturing():
+            return make()
+        at = (torch.device(device), _stream())
+        kept = self._kept.pop(at, None)
+        if kept is None or kept[0] != key:
+            kept = (key, make())
+        self._kept[at] = kept
+        while len(self._kept) > self._most:
+            self._kept.popitem(last=False)
+        return kept[1]
 
 
 _TORCH_DT = {SOP_F32: torch.float32, SOP_BF16: torch.bfloat16, SOP_F16: torch.float16,
@@ -510,26 +543,28 @@ def bake_stats(workspace: BakeWorkspace):
     return int(out[0]), int(out[1]), int(out[2]), int(out[3])
 
 
-_bake_ws = {}
+_bake_ws = _StreamScratch()
 
 
 def bake(gauss, atlas: Atlas, t_near=0.0, alpha_min=1.0 / 255.0, alpha_max=0.99, t_stop=1e-4, workspace=None):
     """Bake every texel of `atlas` against the Gaussians (dict of CUDA
     float32 tensors: mean, scale, quat, opacity, rgb): bin + trace.
     Asynchronous; device_status() reports non-finite inputs or truncated
-    rays."""
-    n = int(gauss["mean"].shape[0])
-    dev = atlas.rgbo.device
-    ws = workspace
-    if ws is None:
-        ws = _bake_ws.get((dev, n))
-        if ws is None:
-            _bake_ws.clear()
-            ws = _bake_ws[(dev, n)] = BakeWorkspace(n, dev)
+    rays. Without a workspace one of the current stream's is kept for the next
+    bake of as many Gaussians; a given workspace serves one bake at a time."""
     g = _gauss(gauss)
     d = atlas.c()
     bp = _bake_params(t_near, alpha_min, alpha_max, t_stop)
-    _check(load().sop_bake(C.byref(g), C.byref(d), C.byref(bp), _ptr(ws.buf), ws.buf.numel(), _stream()))
+
+    def call(ws):
+        _check(load().sop_bake(C.byref(g), C.byref(d), C.byref(bp), _ptr(ws.buf), ws.buf.numel(), _stream()))
+
+    if workspace is not None:
+        call(workspace)
+    else:
+        n, dev = int(gauss["mean"].shape[0]), atlas.rgbo.device
+        with _bake_ws.lock:
+            call(_bake_ws.get(dev, n, lambda: BakeWorkspace(n, dev)))
     return atlas
 
 
@@ -691,7 +726,7 @@ class Surrogate:
                                         C.c_float(self.r_near), C.byref(h), _stream()))
         self._keep = p
         self.h = h
-        self._ws = {}
+        self._ws = _StreamScratch()
 
     def __del__(self):
         try:
@@ -725,11 +760,11 @@ class Surrogate:
         _check(load().sop_surrogate_load(self.h, str(path).encode(), _stream()))
 
     def workspace(self, n_gauss, P, R):
+        """The current stream's scratch for features() and rebake() of these
+        sizes (kept until a call of other sizes on the stream)."""
         key = (int(n_gauss), int(P), int(R))
-        if key not in self._ws:
-            self._ws.clear()
-            self._ws[key] = _ws(int(load().sop_surrogate_workspace_bytes(*key)), self.device)
-        return self._ws[key]
+        return self._ws.get(self.device, key,
+                            lambda: _ws(int(load().sop_surrogate_workspace_bytes(*key)), self.device))
 
     def features(self, gauss, probe_pos, R, alpha_min=1.0 / 255.0, alpha_max=0.99, with_list=False):
         """Texel features [P, R*R, 18] (and the near lists [P, 256] int32)."""
@@ -737,10 +772,11 @@ class Surrogate:
         g = _gauss(gauss)
         feats = torch.empty((P, R * R, self.N_FEATURES), dtype=torch.float32, device=self.device)
         lst = torch.empty((P, self.NEAR_CAP), dtype=torch.int32, device=self.device) if with_list else None
-        ws = self.workspace(g.n, P, R)
         bp = _bake_params(0.0, alpha_min, alpha_max, 1e-4)
-        _check(load().sop_surrogate_features(self.h, C.byref(g), _f32(probe_pos, (P, 3)), P, R, C.byref(bp),
-                                             _ptr(feats), _ptr(lst), _ptr(ws), ws.numel(), _stream()))
+        with self._ws.lock:
+            ws = self.workspace(g.n, P, R)
+            _check(load().sop_surrogate_features(self.h, C.byref(g), _f32(probe_pos, (P, 3)), P, R, C.byref(bp),
+                                                 _ptr(feats), _ptr(lst), _ptr(ws), ws.numel(), _stream()))
         return (feats, lst) if with_list else feats
 
     def train(self, feats, targets: Atlas, steps=1, batch=64, lr=1e-3, seed=0, probe_ids=None, losses=None):
@@ -772,10 +808,11 @@ class Surrogate:
         bp = _bake_params(0.0, alpha_min, alpha_max, t_stop)
         err = torch.empty(1, dtype=torch.float32, device=self.device)
         fell = torch.empty(1, dtype=torch.int32, device=self.device)
-        ws = self.workspace(g.n, out.P, out.R)
-        _check(load().sop_surrogate_infer(self.h, C.byref(g), C.byref(d), C.byref(bp), C.c_float(spot_frac),
-                                          C.c_float(tau), C.c_uint64(seed), _ptr(err), _ptr(fell), _ptr(ws),
-                                          ws.numel(), _stream()))
+        with self._ws.lock:
+            ws = self.workspace(g.n, out.P, out.R)
+            _check(load().sop_surrogate_infer(self.h, C.byref(g), C.byref(d), C.byref(bp), C.c_float(spot_frac),
+                                              C.c_float(tau), C.c_uint64(seed), _ptr(err), _ptr(fell), _ptr(ws),
+                                              ws.numel(), _stream()))
         return err, fell
 
 
