@@ -907,10 +907,7 @@ static cudaError_t adjoint_launch(const AdjK& k, cudaStream_t s)
 {
     const size_t smem = sizeof(float4) * (size_t)k.S;
     auto fn = adjoint_kernel<DT, KMAX>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(fn, smem); e != cudaSuccess) return e;
     fn<<<(unsigned)((k.M + 127) / 128), 128, smem, s>>>(k);
     return cudaGetLastError();
 }
@@ -928,7 +925,7 @@ static cudaError_t adjoint_launch(const AdjK& k, cudaStream_t s)
 constexpr int64_t kAdjSmall = 16384;
 static bool adjoint_by_tile(const AdjK& k)
 {
-    if (adj_smem(k.R, k.S, k.K).total > 220 * 1024) return false;
+    if (adj_smem(k.R, k.S, k.K).total > kSmemMost) return false;
     return k.M <= kAdjSmall || 2 * (int64_t)k.S * k.K >= 3 * (int64_t)point_texels(k.R);
 }
 
@@ -938,7 +935,7 @@ static cudaError_t adjoint_tile_launch(const AdjK& k, cudaStream_t s)
     const size_t smem = adj_smem(k.R, k.S, k.K).total;
     auto fn = adjoint_tile_kernel<DT>;
     int dev = 0, sms = 0;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn, smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;

@@ -1830,10 +1830,7 @@ static cudaError_t shade_launch(const ShadeK& k, int LANES, cudaStream_t s)
     // per-warp direction tables of the shared-normal SHADOW path (8 warps)
     if (MODE == SOP_MODE_SHADOW && k.S <= kShadowTab) smem += (size_t)(bs / 32) * 2 * sizeof(float4) * k.S;
     auto fn = shade_kernel<DT, KMAX, MODE>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(fn, smem); e != cudaSuccess) return e;
     fn<<<nb, bs, smem, s>>>(k, LANES);
     return cudaGetLastError();
 }
@@ -1861,10 +1858,7 @@ static cudaError_t shade_point_launch(const ShadeK& k, cudaStream_t s)
 {
     const size_t smem = sizeof(float4) * (size_t)k.S + kPointWarps * point_smem_bytes(k.R);
     auto fn = shade_point_kernel<DT, KMAX, NR>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(fn, smem); e != cudaSuccess) return e;
     fn<<<(unsigned)((k.M + kPointWarps - 1) / kPointWarps), kPointWarps * 32, smem, s>>>(k);
     return cudaGetLastError();
 }
@@ -1893,7 +1887,7 @@ static bool shade_by_point(const QueryArgs& a)
 {
     if (a.mode != SOP_MODE_SHADE || a.dir_world) return false;
     const int64_t t = point_texels(a.R), sk = (int64_t)a.S * a.K;
-    if (sizeof(float4) * (size_t)a.S + kPointWarps * point_smem_bytes(a.R) > 220 * 1024) return false;
+    if (sizeof(float4) * (size_t)a.S + kPointWarps * point_smem_bytes(a.R) > kSmemMost) return false;
     return sk >= (a.rgbo_dtype == SOP_F32 ? 3 : 4) * t || (a.M <= kPointSmall && sk >= t);
 }
 
@@ -1927,10 +1921,7 @@ static cudaError_t shade_world_launch(const ShadeK& k, cudaStream_t s)
     const unsigned nb = (unsigned)((threads + bs - 1) / bs);
     const size_t smem = 3 * sizeof(float4) * (size_t)k.S;
     auto fn = shade_world_kernel<DT, KMAX, MODE>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(fn, smem); e != cudaSuccess) return e;
     fn<<<nb, bs, smem, s>>>(k, LANES);
     return cudaGetLastError();
 }
@@ -2340,10 +2331,7 @@ static cudaError_t shade_direct_launch(const ShadeDirectK& k, cudaStream_t s)
 {
     const size_t smem = sizeof(float4) * (size_t)k.S;
     auto fn = shade_direct_kernel<DT, KMAX, MODE>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem(fn, smem); e != cudaSuccess) return e;
     fn<<<(unsigned)((k.M + 255) / 256), 256, smem, s>>>(k);
     return cudaGetLastError();
 }

@@ -177,6 +177,18 @@ unsigned int* status_word();
 cudaError_t status_take(uint32_t* host_out, bool clear, cudaStream_t s);
 const char* status_bits_message(uint32_t bits);
 
+// Dynamic shared memory of a kernel whose need varies from call to call. The
+// limit is a property of the kernel, not of the launch, so it is set to one
+// value for all calls: set to each call's own need, another host thread's call
+// with less could lower it before the launch, which would then be refused.
+constexpr size_t kSmemMost = 220 * 1024;
+template <class Kernel>
+inline cudaError_t allow_smem(Kernel* fn, size_t need)
+{
+    if (need <= 40 * 1024) return cudaSuccess;  // (48 KB, static included, need no leave)
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost);
+}
+
 inline size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 }  // namespace sop

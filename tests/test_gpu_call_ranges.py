@@ -101,3 +101,67 @@ def test_coarsened_bakes(sop, orc, n, length, width, two, extra):
     assert_close(occ[decided], o_occ[decided], what="O", absolute=sens[..., 3][decided])
     ok = decided & ((fl & orc.FLAG_ORDER) == 0)
     assert_close(rgb[ok], o_rgb[ok], what="L_in", absolute=sens[..., :3][ok])
+
+
+def test_bakes_on_two_streams(sop):
+    """Bakes of equally many Gaussians side by side on two streams, each with
+    its stream's own scratch: the maps of single bakes, bit for bit."""
+    pp = cuda(np.random.default_rng(1).uniform(-1, 1, (256, 3)).astype(F))
+    sets = [{k: cuda(v) for k, v in _rods(20_000, 0.02, 0.01, False, seed).items()} for seed in (3, 4)]
+    want = [sop.make_atlas(pp, 8) for _ in sets]
+    for g, at in zip(sets, want):
+        sop.bake(g, at)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in sets]
+    got = [[sop.make_atlas(pp, 8) for _ in range(10)] for _ in sets]
+    torch.cuda.synchronize()
+    for i in range(10):
+        for s, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                sop.bake(sets[s], got[s][i])
+    torch.cuda.synchronize()
+    for s in range(2):
+        for at in got[s]:
+            assert torch.equal(at.rgbo, want[s].rgbo) and torch.equal(at.depth, want[s].depth)
+
+
+def test_queries_of_several_threads(sop):
+    """Host threads with maps and direction sets of different sizes, whose
+    launches want different amounts of shared memory of the same kernels:
+    every call is accepted, and returns what it returns alone."""
+    import threading
+    rng = np.random.default_rng(5)
+    M, K = 48, 8
+    x, n = rng.uniform(-1, 1, (M, 3)).astype(F), rng.standard_normal((M, 3))
+    n = (n / np.linalg.norm(n, axis=1, keepdims=True)).astype(F)
+    pts = [cuda(v) for v in (x, n, n, rng.uniform(0, 1, (M, 3)).astype(F), np.full(M, 0.5, F), np.full(M, 0.5, F))]
+    env, go = cuda(rng.uniform(0.5, 1, (8, 16, 3)).astype(F)), cuda(rng.standard_normal((M, 3)).astype(F))
+    jobs = []
+    for R, S in ((16, 128), (24, 128), (18, 700), (8, 4096)):
+        P = 16
+        at = sop.make_atlas(cuda(rng.uniform(-1, 1, (P, 3)).astype(F)), R, with_depth=False)
+        sop.atlas_pack(cuda(rng.uniform(0, 0.5, (P, R, R, 3)).astype(F)), cuda(rng.uniform(0, 1, (P, R, R)).astype(F)), None, at)
+
+        def job(at=at, S=S):
+            out = sop.query_shade(*pts, at, env, K, S)
+            return [out] + [sop.query_shade_backward(*pts, at, env, K, S, go)[k] for k in ("albedo", "rough", "normal")]
+        jobs.append((job, [t.clone() for t in job()]))
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(job, want):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(300):
+                    got = job()
+                torch.cuda.current_stream().synchronize()
+                if not all(torch.equal(a, b) for a, b in zip(got, want)):
+                    failed.append("other results")
+        except Exception as e:  # a refused launch
+            failed.append(repr(e))
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
