@@ -974,6 +974,7 @@ struct DirTerms {
     float3 w;
     float2 uv;
     int off;
+    float fu, fv;
     float w00, w10, w01, w11;
 };
 // footprint part for a world direction w
@@ -988,6 +989,8 @@ __device__ __forceinline__ DirTerms footprint_terms(const float3 w, const float 
     const float fu = s - fi, fv = t - fj;
     const int i0 = min(max((int)fi + 1, 0), R), j0 = min(max((int)fj + 1, 0), R);
     d.off = j0 * RQ + i0;
+    d.fu = fu;
+    d.fv = fv;
     d.w00 = (1.f - fu) * (1.f - fv);
     d.w10 = fu * (1.f - fv);
     d.w01 = (1.f - fu) * fv;
@@ -1237,10 +1240,15 @@ __global__ void __launch_bounds__(256, 4) shade_kernel(const ShadeK a, const int
 // ---------------------------------------------------------------------------
 // SHADOW mode, large calls: one thread per point.
 //
-// The shadow ratio is 1 - sum_i L_i cos_i O(w_i) / sum_i L_i cos_i with O =
+// The shadow ratio is sum_i L_i cos_i (1 - O(w_i)) / sum_i L_i cos_i with O =
 // sum_k W_k O_k (Eq. 5 applied to O), so the sum over directions can be taken
-// per probe first: V_k = sum_i L_i cos_i O_k(w_i), ratio = 1 - sum_k W_k V_k /
-// den. V_k depends on the point only through its normal. Where the points of
+// per probe first: V_k = sum_i L_i cos_i (1 - O_k(w_i)), and over the probes
+// what is visible, num = sum_k W_k V_k, and what is hidden, hid = sum_k W_k (den
+// - V_k): the ratio is num / (num + hid), taken from the smaller of the two, so
+// that what is left of a hidden light is no difference of large sums and a
+// point that nothing hides is exactly 1. (The weights' sum is 1 but for its
+// rounding, which cancels.) V_k depends on the point only through its normal.
+// Where the points of
 // a warp share one normal bit for bit (a planar receiver such as a ground
 // plane: their directions, footprints and environment terms coincide), the
 // warp takes each of its distinct probes once, the lanes over the directions,
@@ -1257,6 +1265,9 @@ constexpr int kShadowProbes = 32;
 // float32 on an object 284 / 274; 2,051,693 on a ground: 1,240 / 776. A warp's
 // few serial steps do not fill the machine below.
 constexpr int64_t kShadowWarpPoints = 262144;
+// Up to 16 probes a point: 32 spill (1,000,000 ground points, K 32, whole call:
+// 3,614 us in lanes, 4,025 here; K 16: 1,328 / 955).
+constexpr int kShadowWarpK = 16;
 
 // Ratio of one point by blending per direction, LANES threads a point.
 template <int DT, int KMAX, int LANES>
@@ -1305,7 +1316,8 @@ __device__ __forceinline__ void shadow_point(const ShadeK& a, const float4* __re
         for (int c = 0; c < 3; ++c) a.out[3 * m + c] = den[c] < 1e-20f ? 1.f : acc[c] / den[c];
 }
 
-template <int DT, int KMAX>
+// LANES: threads a point of the warps without a common normal (shade_lanes)
+template <int DT, int KMAX, int LANES>
 __global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
 {
     extern __shared__ float4 s_dirs[];
@@ -1367,8 +1379,8 @@ __global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
                     const float3 Ld = a.env_layout == SOP_ENV_OCTAHEDRAL ? env_oct_lookup(a.envq, a.He, d.uv)
                                                                          : env_lookup(a.envq, a.He, a.We, d.w);
                     off[r] = d.off;
-                    fu[r] = d.w10 + d.w11;
-                    fv[r] = d.w01 + d.w11;
+                    fu[r] = d.fu;
+                    fv[r] = d.fv;
                     L[r][0] = Ld.x * l.z;
                     L[r][1] = Ld.y * l.z;
                     L[r][2] = Ld.z * l.z;
@@ -1376,9 +1388,14 @@ __global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
                     for (int c = 0; c < 3; ++c) den[c] += L[r][c];
                 }
             }
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) den[c] += __shfl_xor_sync(full, den[c], o);
             // two probes a step: their loads overlap, and the sums over the
-            // lanes go on in one half of the warp each
-            float num[3] = {0.f, 0.f, 0.f};
+            // lanes go on in one half of the warp each (in the order of den's,
+            // so that a probe that hides nothing has V = den)
+            float num[3] = {0.f, 0.f, 0.f}, hid[3] = {0.f, 0.f, 0.f};
             const bool lower = lane < 16;
             for (int u = 0; u < n; u += 2) {
                 int32_t p[2];
@@ -1396,11 +1413,11 @@ __global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
                         const float4 qb = OQuad<DT>::load(a.quads, (int64_t)(p[1] * RQ * RQ + off[r]));
                         const float la = fmaf(fu[r], qa.y - qa.x, qa.x), ha = fmaf(fu[r], qa.w - qa.z, qa.z);
                         const float lb = fmaf(fu[r], qb.y - qb.x, qb.x), hb = fmaf(fu[r], qb.w - qb.z, qb.z);
-                        const float Oa = fmaf(fv[r], ha - la, la), Ob = fmaf(fv[r], hb - lb, lb);
+                        const float va = 1.f - fmaf(fv[r], ha - la, la), vb = 1.f - fmaf(fv[r], hb - lb, lb);
 #pragma unroll
                         for (int c = 0; c < 3; ++c) {
-                            V[0][c] = fmaf(L[r][c], Oa, V[0][c]);
-                            V[1][c] = fmaf(L[r][c], Ob, V[1][c]);
+                            V[0][c] = fmaf(L[r][c], va, V[0][c]);
+                            V[1][c] = fmaf(L[r][c], vb, V[1][c]);
                         }
                     }
 #pragma unroll
@@ -1414,22 +1431,27 @@ __global__ void __launch_bounds__(256, 4) shadow_warp_kernel(const ShadeK a)
                     float v = (lower ? V[0][c] : V[1][c]) + __shfl_xor_sync(full, lower ? V[1][c] : V[0][c], 16);
 #pragma unroll
                     for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
-                    const float x = __shfl_xor_sync(full, v, 16);
-                    if (w[0] != 0.f) num[c] = fmaf(w[0], lower ? v : x, num[c]);
-                    if (w[1] != 0.f) num[c] = fmaf(w[1], lower ? x : v, num[c]);
+                    const float x = __shfl_xor_sync(full, v, 16), va = lower ? v : x, vb = lower ? x : v;
+                    if (w[0] != 0.f) {
+                        num[c] = fmaf(w[0], va, num[c]);
+                        hid[c] = fmaf(w[0], den[c] - va, hid[c]);
+                    }
+                    if (w[1] != 0.f) {
+                        num[c] = fmaf(w[1], vb, num[c]);
+                        hid[c] = fmaf(w[1], den[c] - vb, hid[c]);
+                    }
                 }
             }
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) den[c] += __shfl_xor_sync(full, den[c], o);
-                if (active) a.out[3 * m + c] = den[c] < 1e-20f ? 1.f : (den[c] - num[c]) / den[c];
+                // (no probe found: both sums are 0, nothing hides the point)
+                const float sum = num[c] + hid[c];
+                const float ratio = hid[c] <= num[c] ? 1.f - (hid[c] != 0.f ? hid[c] / sum : 0.f) : num[c] / sum;
+                if (active) a.out[3 * m + c] = den[c] < 1e-20f ? 1.f : ratio;
             }
             return;
         }
     }
-    // as many lanes a point as shade_kernel takes
-    constexpr int LANES = DT == SOP_F32 ? 1 : 2;
     for (int j = 0; j < LANES; ++j) {
         const int64_t mj = m0 + j * (32 / LANES) + lane / LANES;
         shadow_point<DT, KMAX, LANES>(a, s_dirs, mj, lane % LANES, mj < a.M);
@@ -1891,21 +1913,27 @@ static bool shade_by_point(const QueryArgs& a)
     return sk >= (a.rgbo_dtype == SOP_F32 ? 3 : 4) * t || (a.M <= kPointSmall && sk >= t);
 }
 
-template <int DT, int KMAX>
+template <int DT, int KMAX, int LANES>
 static cudaError_t shadow_warp_launch(const ShadeK& k, cudaStream_t s)
 {
-    shadow_warp_kernel<DT, KMAX><<<(unsigned)((k.M + 255) / 256), 256, sizeof(float4) * (size_t)k.S, s>>>(k);
+    shadow_warp_kernel<DT, KMAX, LANES><<<(unsigned)((k.M + 255) / 256), 256, sizeof(float4) * (size_t)k.S, s>>>(k);
     return cudaGetLastError();
+}
+template <int DT, int KMAX>
+static cudaError_t shadow_warp_dispatch(const ShadeK& k, cudaStream_t s)
+{
+    // (kShadowWarpPoints leaves one or two)
+    if (DT == SOP_F32 && shade_lanes(DT, k.M) == 1) return shadow_warp_launch<DT, KMAX, 1>(k, s);
+    return shadow_warp_launch<DT, KMAX, 2>(k, s);
 }
 
 template <int DT, int MODE>
 static cudaError_t shade_k(const ShadeK& k, cudaStream_t s)
 {
-    if (MODE == SOP_MODE_SHADOW && k.S <= kShadowTab && k.M >= kShadowWarpPoints) {
-        if (k.K <= 4) return shadow_warp_launch<DT, 4>(k, s);
-        if (k.K <= 8) return shadow_warp_launch<DT, 8>(k, s);
-        if (k.K <= 16) return shadow_warp_launch<DT, 16>(k, s);
-        return shadow_warp_launch<DT, 32>(k, s);
+    if (MODE == SOP_MODE_SHADOW && k.S <= kShadowTab && k.M >= kShadowWarpPoints && k.K <= kShadowWarpK) {
+        if (k.K <= 4) return shadow_warp_dispatch<DT, 4>(k, s);
+        if (k.K <= 8) return shadow_warp_dispatch<DT, 8>(k, s);
+        return shadow_warp_dispatch<DT, 16>(k, s);
     }
     if (k.K <= 4) return shade_dispatch<DT, 4, MODE>(k, s);
     if (k.K <= 8) return shade_dispatch<DT, 8, MODE>(k, s);

@@ -165,3 +165,59 @@ def test_queries_of_several_threads(sop):
     for t in threads:
         t.join()
     assert not failed, failed
+
+
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_shadow_of_a_hidden_sun(sop, orc, dtype):
+    """A large SHADOW call on one plane whose only bright light is hidden by
+    its probe: what is left is a small sum, not the difference of two large
+    ones. One probe a point (its weight is exactly 1). Bound: 1e-5 and the
+    sensitivity to the rounding of the directions."""
+    M, P, R, S, He = 262_144, 40, 8, 64, 16
+    rng = np.random.default_rng(11)
+    pp = np.concatenate([rng.uniform(-1, 1, (P, 2)), np.full((P, 1), 0.05)], axis=1).astype(F)
+    x = np.concatenate([rng.uniform(-1, 1, (M, 2)), np.zeros((M, 1))], axis=1).astype(F)
+    n = np.tile(np.array([0.0, 0.0, 1.0], F), (M, 1))
+    env = rng.uniform(0.005, 0.015, (He, 2 * He, 3)).astype(F)
+    r, c = 4, 9  # a sun half way up
+    env[r:r + 2, c:c + 2] = 2e4
+    th, ph = (r + 1) / He * np.pi, (c + 1) / He * np.pi - np.pi
+    sun = np.array([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)])
+    u = (np.arange(R) + 0.5) / R * 2 - 1
+    px, py = np.meshgrid(u, u, indexing="xy")
+    z = 1 - np.abs(px) - np.abs(py)
+    fx, fy = (np.where(z < 0, (1 - np.abs(b)) * np.where(a >= 0, 1, -1), a) for a, b in ((px, py), (py, px)))
+    d = np.stack([fx, fy, z], -1)
+    d /= np.linalg.norm(d, axis=-1, keepdims=True)
+    occ = np.where(d @ sun > np.cos(np.deg2rad(75)), 1.0, rng.integers(0, 33, (P, R, R)) / 64).astype(F)
+    rgb, one = np.zeros((P, R, R, 3), F), np.full(M, 0.5, F)
+    at = sop.make_atlas(cuda(pp), R, dtype, with_depth=False)
+    sop.atlas_pack(cuda(rgb), cuda(occ), None, at)
+    out = sop.query_shade(*[cuda(v) for v in (x, n, n, np.full((M, 3), 0.5, F), one, one)], at, cuda(env), 1, S,
+                          mode=sop.MODE_SHADOW).cpu().numpy()
+    sel = rng.integers(0, M, 200)
+    args = [x[sel], n[sel], n[sel], np.full((200, 3), 0.5, F), one[sel], one[sel], pp, rgb, occ, env, 1, S]
+    want, _, _ = orc.query_shade(*args, mode=orc.MODE_SHADOW)
+    sens = orc.query_shade_sensitivity(*args, mode=orc.MODE_SHADOW)
+    assert 0 < want.max() < 1e-3
+    assert np.all(np.abs(out[sel] - want) <= 1e-5 * np.maximum(np.abs(want), 1e-3 * np.abs(want).mean()) + sens)
+
+
+@pytest.mark.parametrize("K,radius", [(5, 0.0), (9, 0.0), (17, 0.0), (6, 0.01)])
+@pytest.mark.parametrize("M", [262_144, 311_296])
+def test_shadow_of_nothing(sop, K, radius, M):
+    """Probes that hide nothing, and points with no probe within the radius:
+    the ratio is exactly 1, also where a warp's points share their sums."""
+    rng = np.random.default_rng(K)
+    P, R = 64, 8
+    pp = np.concatenate([rng.uniform(-1, 1, (P, 2)), np.full((P, 1), 0.02)], axis=1).astype(F)
+    x = np.zeros((M, 3), F)
+    x[:, 0] = np.linspace(-1.2, 1.2, M)
+    n = np.tile(np.array([0.0, 0.0, 1.0], F), (M, 1))
+    at = sop.make_atlas(cuda(pp), R, with_depth=False)
+    sop.atlas_pack(cuda(np.zeros((P, R, R, 3), F)), cuda(np.zeros((P, R, R), F)), None, at)
+    env = np.exp(rng.normal(0, 1.5, (16, 32, 3))).astype(F)
+    one = np.full(M, 0.5, F)
+    out = sop.query_shade(*[cuda(v) for v in (x, n, n, np.full((M, 3), 0.5, F), one, one)], at, cuda(env), K, 64,
+                          mode=sop.MODE_SHADOW, radius=radius)
+    assert bool((out == 1).all())
