@@ -1895,22 +1895,41 @@ static cudaError_t shade_point_k(const ShadeK& k, cudaStream_t s)
 }
 
 // Which SHADE kernel: a warp a point pays for the texels that its directions
-// touch ((R+2)^2 stored, about half of them), then little a direction; a
-// thread a point (or a few lanes) pays K footprints a direction. Measured on
-// 418,111 points of a view, us a call (lanes / warp): float32, R 16, K 8:
-// S 128 1,998 / 1,683, S 64 1,153 / 1,305; K 4, S 128 1,116 / 1,335; R 8, K 8:
-// S 128 1,938 / 1,423, S 32 697 / 902; R 24, S 128 2,041 / 2,939; 16 bits,
-// R 16, S 128 1,575 / 1,548. 50,000 points, S 512: 1,733 / 621. So S K has to
-// reach 3 (4 at 16 bits) times the texels. Small calls do not fill the
-// machine with a thread a point: 21,907 points, S 64: 276 / 220; 1,000: 204 /
-// 170.
+// touch ((R+2)^2 stored, about half of them) and a fixed amount, then little a
+// direction; a thread a point (or a few lanes) pays K footprints a direction.
+// Measured on views, us a call (lanes / warp). 418,111 points: float32, R 16,
+// K 8: S 128 1,998 / 1,683, S 64 1,153 / 1,305; K 4, S 128 1,116 / 1,335; R 8,
+// K 8: S 128 1,938 / 1,423, S 32 697 / 902; R 24, S 128 2,041 / 2,939; 16 bits,
+// R 16, S 128 1,575 / 1,548. So S K has to reach 3 (4 at 16 bits) times the
+// texels. Small maps leave the fixed amount, more than a few probes' footprints
+// from near caches: 300,000 points, R 2: K 4: S 32 262 / 431, S 128 695 / 809,
+// K 8: S 64 682 / 615 (float32), 554 / 605 (16 bits), K 16, S 64 1,006 / 802;
+// 1,000,000 points, float32, R 4, K 4, S 400: 5,313 / 6,922. Where the lanes
+// are several a point, sharing its footprints' addresses costs them more:
+// 100,000 points, float32, R 8, K 4, S 64: 262 / 232; S 128: 444 / 311; 60,000
+// points, 16 bits, R 8, K 8, S 64: 203 / 190. (More than 128 directions have
+// their footprints computed twice: 300,000 points, float32, R 4, K 4, S 400:
+// 1,959 / 2,142, R 8: 2,087 / 1,937.)
+// Calls of few points do not fill the machine with a thread a point: 21,907
+// points, S 64: 276 / 220; 1,000: 204 / 170; and the fewer, the less a warp has
+// to save (R 3, K 1, S 32: 16,384 points 72 / 83, 32,768: 83 / 103).
 constexpr int64_t kPointSmall = 32768;
 static bool shade_by_point(const QueryArgs& a)
 {
     if (a.mode != SOP_MODE_SHADE || a.dir_world) return false;
-    const int64_t t = point_texels(a.R), sk = (int64_t)a.S * a.K;
-    if (sizeof(float4) * (size_t)a.S + kPointWarps * point_smem_bytes(a.R) > kSmemMost) return false;
-    return sk >= (a.rgbo_dtype == SOP_F32 ? 3 : 4) * t || (a.M <= kPointSmall && sk >= t);
+    const int64_t t = point_texels(a.R), S = a.S, sk = S * a.K;
+    if (sizeof(float4) * (size_t)S + kPointWarps * point_smem_bytes(a.R) > kSmemMost) return false;
+    const bool f32 = a.rgbo_dtype == SOP_F32;
+    if (a.M <= kPointSmall) {
+        const int64_t least = f32 ? (a.M < 7500 ? a.M / 50 : 150) : a.M / 64;
+        return sk >= t && sk >= least;
+    }
+    if (sk < (f32 ? 3 : 4) * t) return false;
+    const int lanes = shade_lanes(a.rgbo_dtype, a.M);
+    if (f32 && lanes >= 4) return sk >= 150;
+    if (!f32 && lanes >= 8) return sk - S >= 400;
+    if (f32 && lanes == 2) return sk - (S > 128 && t < 64 ? 4 : 2) * S >= 300;
+    return sk - 3 * S >= 400 + t / 2;
 }
 
 template <int DT, int KMAX, int LANES>

@@ -221,3 +221,36 @@ def test_shadow_of_nothing(sop, K, radius, M):
     out = sop.query_shade(*[cuda(v) for v in (x, n, n, np.full((M, 3), 0.5, F), one, one)], at, cuda(env), K, 64,
                           mode=sop.MODE_SHADOW, radius=radius)
     assert bool((out == 1).all())
+
+
+@pytest.mark.parametrize("R,M,K,S,dtype", [
+    (2, 33_000, 4, 32, 0), (2, 33_000, 4, 40, 0),            # float32, several lanes: S K = 150
+    (2, 160_000, 4, 128, 0), (2, 160_000, 5, 104, 0),        # two lanes: S (K - 2) = 300
+    (3, 160_000, 4, 400, 0), (3, 160_000, 6, 400, 0),
+    (2, 33_000, 5, 99, 2), (2, 33_000, 5, 100, 1),           # 16 bits, eight lanes: S (K - 1) = 400
+    (2, 80_000, 6, 135, 1), (2, 80_000, 6, 137, 2),          # fewer: S (K - 3) = 400 + texels / 2
+    (3, 1000, 1, 32, 0), (3, 16_384, 1, 32, 0), (3, 16_384, 8, 32, 1),  # few points
+])
+def test_shade_dispatch(sop, orc, R, M, K, S, dtype):
+    """SHADE on both sides of the lines between its kernels on small maps (in
+    which a footprint of texels is most of the map): a sample against the oracle,
+    with the bound of the query's other tests, on maps that are exact in 16 bits."""
+    rng = np.random.default_rng(R * M + S)
+    P = 40
+    pp, x = rng.uniform(-1, 1, (P, 3)).astype(F), rng.uniform(-1, 1, (M, 3)).astype(F)
+    n = rng.standard_normal((M, 3))
+    wo = rng.standard_normal((M, 3))
+    wo *= np.sign(np.sum(wo * n, axis=1, keepdims=True))
+    n, wo = ((v / np.linalg.norm(v, axis=1, keepdims=True)).astype(F) for v in (n, wo))
+    th, ph = (np.arange(16) + 0.5) / 16 * np.pi, (np.arange(32) + 0.5) / 16 * np.pi
+    env = (1.0 + 0.5 * np.sin(th)[:, None, None] * np.cos(ph[None, :, None] + np.arange(3))).astype(F)
+    rgb, occ = ((rng.integers(0, 65, s) / 64).astype(F) for s in ((P, R, R, 3), (P, R, R)))
+    pts = (x, n, wo, rng.uniform(0, 1, (M, 3)).astype(F), rng.uniform(0.3, 1, M).astype(F), rng.uniform(0, 1, M).astype(F))
+    at = sop.make_atlas(cuda(pp), R, dtype, with_depth=False)
+    sop.atlas_pack(cuda(rgb), cuda(occ), None, at)
+    out = sop.query_shade(*[cuda(v) for v in pts], at, cuda(env), K, S).cpu().numpy()
+    sel = np.unique(np.concatenate([rng.integers(0, M, 100), np.arange(M - 40, M)]))
+    args = [v[sel] for v in pts] + [pp, rgb, occ, env, K, S]
+    want, _, _ = orc.query_shade(*args)
+    sens = orc.query_shade_sensitivity(*args)
+    assert np.all(np.abs(out[sel] - want) <= 1e-5 * np.maximum(np.abs(want), 1e-3 * np.abs(want).mean()) + sens)
