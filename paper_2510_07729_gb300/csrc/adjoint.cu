@@ -918,15 +918,25 @@ static cudaError_t adjoint_launch(const AdjK& k, cudaStream_t s)
 // Measured at R = 16 on 418,111 points of a view, us a call (thread / tile):
 // S 128, K 8: 12,680 / 7,270; S 64, K 8: 6,760 / 5,460; S 32, K 8: 3,850 /
 // 4,420; S 32, K 4: 2,220 / 3,430. R = 24, 100,000 points: S 128: 3,630 /
-// 3,750, S 32: 1,120 / 2,270. So the line lies near S K = 1.5 (R+2)^2. A
+// 3,750, S 32: 1,120 / 2,270. So the line lies near S K = 1.5 (R+2)^2, and on
+// small maps near S (K + 4) = 100 (60,000 points, R 2, K 4, S 8: 280 / 354). A
 // thread takes its S directions one after the other, about 8 us each however
 // few points there are, so small calls go to the tile kernel (1,000 points,
-// S 128: 1,080 / 310; 8,191 points: 1,060 / 450).
+// S 128: 1,080 / 310; 8,191 points: 1,060 / 450) unless they have few
+// directions: the line rises with the points, and twice as fast where an SM
+// holds one CTA instead of two (16,384 points, K 4: R 8: S 16 177 / 189, S 32 229
+// / 196; R 16: S 32 224 / 228, S 64 345 / 267; R 24: S 8 130 / 285, S 64 342 /
+// 440).
 constexpr int64_t kAdjSmall = 16384;
+constexpr size_t kAdjTwoCtas = 110 * 1024;  // shared memory of two CTAs an SM
 static bool adjoint_by_tile(const AdjK& k)
 {
-    if (adj_smem(k.R, k.S, k.K).total > kSmemMost) return false;
-    return k.M <= kAdjSmall || 2 * (int64_t)k.S * k.K >= 3 * (int64_t)point_texels(k.R);
+    const size_t smem = adj_smem(k.R, k.S, k.K).total;
+    if (smem > kSmemMost) return false;
+    const int64_t t = point_texels(k.R), sk = (int64_t)k.S * k.K;
+    const int64_t least = (100 + 3 * t / 5) * (smem <= kAdjTwoCtas ? 1 : 2);
+    if (k.M <= kAdjSmall) return (sk + 4 * (int64_t)k.S) * kAdjSmall >= least * k.M;
+    return 2 * sk >= 3 * t && sk + 4 * (int64_t)k.S >= least;
 }
 
 template <int DT>
@@ -940,7 +950,7 @@ static cudaError_t adjoint_tile_launch(const AdjK& k, cudaStream_t s)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     // two CTAs an SM (their registers' limit) where shared memory holds both
-    const int64_t tiles = (k.M + kAdjPts - 1) / kAdjPts, most = (int64_t)sms * (smem <= 110 * 1024 ? 2 : 1);
+    const int64_t tiles = (k.M + kAdjPts - 1) / kAdjPts, most = (int64_t)sms * (smem <= kAdjTwoCtas ? 2 : 1);
     fn<<<(unsigned)(tiles < most ? tiles : most), kAdjPts * 32, smem, s>>>(k);
     return cudaGetLastError();
 }

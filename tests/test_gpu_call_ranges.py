@@ -254,3 +254,41 @@ def test_shade_dispatch(sop, orc, R, M, K, S, dtype):
     want, _, _ = orc.query_shade(*args)
     sens = orc.query_shade_sensitivity(*args)
     assert np.all(np.abs(out[sel] - want) <= 1e-5 * np.maximum(np.abs(want), 1e-3 * np.abs(want).mean()) + sens)
+
+
+@pytest.mark.parametrize("R,M,K,S", [
+    (24, 16_384, 4, 64), (24, 4096, 4, 40), (24, 4096, 2, 20), (16, 16_384, 4, 36), (16, 16_384, 4, 37),
+    (8, 16_384, 4, 20), (8, 16_385, 4, 38), (8, 16_385, 12, 9), (2, 16_385, 4, 13), (2, 16_385, 4, 14),
+    (16, 16_385, 17, 29), (64, 300, 16, 24), (64, 300, 32, 12),
+])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_adjoint_dispatch(sop, orc, R, M, K, S, dtype):
+    """The adjoint on both sides of the lines between its kernels, every type of
+    atlas and number of probes in each: a sample's own gradients, and for few
+    points the summed ones, against the oracle, on maps that are exact in 16
+    bits, with the tolerances of the adjoint's other tests."""
+    rng = np.random.default_rng(R * M + S)
+    P = 40
+    pp, x = rng.uniform(-1, 1, (P, 3)).astype(F), rng.uniform(-1, 1, (M, 3)).astype(F)
+    n = rng.standard_normal((M, 3))
+    wo = rng.standard_normal((M, 3))
+    wo *= np.sign(np.sum(wo * n, axis=1, keepdims=True))
+    n, wo = ((v / np.linalg.norm(v, axis=1, keepdims=True)).astype(F) for v in (n, wo))
+    th, ph = (np.arange(16) + 0.5) / 16 * np.pi, (np.arange(32) + 0.5) / 16 * np.pi
+    env = (1.0 + 0.5 * np.sin(th)[:, None, None] * np.cos(ph[None, :, None] + np.arange(3))).astype(F)
+    rgb, occ = ((rng.integers(0, 65, s) / 64).astype(F) for s in ((P, R, R, 3), (P, R, R)))
+    pts = (x, n, wo, rng.uniform(0, 1, (M, 3)).astype(F), rng.uniform(0.3, 1, M).astype(F), rng.uniform(0, 1, M).astype(F))
+    go = rng.standard_normal((M, 3)).astype(F)
+    at = sop.make_atlas(cuda(pp), R, dtype, with_depth=False)
+    sop.atlas_pack(cuda(rgb), cuda(occ), None, at)
+    g = sop.query_shade_backward(*[cuda(v) for v in pts], at, cuda(env), K, S, cuda(go))
+    sel = np.arange(M) if M <= 300 else np.unique(np.concatenate([rng.integers(0, M, 100), np.arange(M - 40, M)]))
+    w = orc.query_shade_grad(*[v[sel] for v in pts], pp, rgb, occ, env, K, S, go[sel])
+    for key in ("albedo", "rough", "metal", "normal"):
+        d = np.abs(g[key].cpu().numpy()[sel] - w[key])
+        terms = w["abs_" + key][:, None] if key == "normal" else w["abs_" + key]
+        assert np.all(d <= 1e-4 * np.abs(w[key]) + 2e-4 * terms + 1e-12), key
+    if M <= 300:
+        for got, ref in ((g["env"], w["env"]), (g["maps"][..., :3], w["maps_rgb"]), (g["maps"][..., 3], w["maps_occ"])):
+            d = np.abs(got.cpu().numpy() - ref)
+            assert np.all(d <= 1e-4 * np.abs(ref) + 2e-5 * np.abs(ref).max() + 1e-12)
