@@ -118,6 +118,8 @@ __global__ void __launch_bounds__(kImpThreads) imp_sample_kernel(const ImpK k)
     constexpr int NW = kImpThreads / 32, PER = kImpMaxTiles / kImpThreads, RND = kImpTile / 128;
     __shared__ int64_t s_cum[kImpMaxTiles];  // inclusive sums of the tiles
     __shared__ int64_t s_w[NW];
+    __shared__ int64_t s_at[NW];  // the warps' texels and their q
+    __shared__ int32_t s_q[NW];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t v[PER], sum = 0;
@@ -140,8 +142,7 @@ __global__ void __launch_bounds__(kImpThreads) imp_sample_kernel(const ImpK k)
 #pragma unroll
     for (int j = 0; j < PER; ++j) s_cum[threadIdx.x * PER + j] = base + v[j];
     __syncthreads();
-    const int i = blockIdx.x * NW + warp;
-    if (i >= k.S) return;
+    const int i = min((int)(blockIdx.x * NW) + warp, k.S - 1);
     const int64_t Q = s_cum[k.n_tiles - 1];
     const int64_t target = (2 * (int64_t)i + 1) * Q / (2 * (int64_t)k.S);
     int lo = 0, hi = k.n_tiles - 1;  // smallest tile whose inclusive sum exceeds the target
@@ -183,11 +184,19 @@ __global__ void __launch_bounds__(kImpThreads) imp_sample_kernel(const ImpK k)
         q = __shfl_sync(full, q, win);
         break;
     }
-    if (lane != 0) return;
+    // the direction and density in double, a lane a sample of the CTA's
+    if (lane == 0) {
+        s_at[warp] = at;
+        s_q[warp] = q;
+    }
+    __syncthreads();
+    const int o = blockIdx.x * NW + lane;
+    if (warp != 0 || lane >= NW || o >= k.S) return;
+    at = s_at[lane];
     double d[3];
     oct_decode_centre_f64(k.H, (int)(at % k.H), (int)(at / k.H), d);
-    const double pdf = (double)k.T * (double)q / (4.0 * 3.14159265358979323846 * (double)Q);
-    k.out[i] = make_float4((float)d[0], (float)d[1], (float)d[2], (float)pdf);
+    const double pdf = (double)k.T * (double)s_q[lane] / (4.0 * 3.14159265358979323846 * (double)Q);
+    k.out[o] = make_float4((float)d[0], (float)d[1], (float)d[2], (float)pdf);
 }
 
 size_t importance_ws_bytes(int32_t H)
