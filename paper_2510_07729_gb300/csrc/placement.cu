@@ -28,8 +28,10 @@
 // 750,710 points, 4,096 choices: 73.1 ms with one choice a link in one
 // 16-CTA cluster whose slices lay in L2; 26.6 ms with the points in the
 // registers of all SMs and one choice a link, every CTA polling every other
-// (the polls crowd L2); 2.0 ms as described (395 links of about 10,000
-// cycles: a third the leader's ranking, a third the two exchanges).
+// (the polls crowd L2); 1.69 to 1.79 ms as described (395 links of about 9,000
+// cycles: a third the leader's ranking, a third the two exchanges). On a
+// lattice, where ties leave one choice a link, 10,648 points and 4,096 choices
+// take 12.0 ms (22.0 in the cluster).
 #include <climits>
 
 #include "scan.cuh"
@@ -43,7 +45,7 @@ constexpr int kFpsWarps = kFpsThreads / 32;
 constexpr int kFpsMaxCtas = 160;
 constexpr int kFpsPicks = 32;   // choices a link at most (one a lane)
 constexpr int kFpsCopies = 8;   // of the list of choices, to spread its readers
-constexpr int kFpsRegPoints = 512;  // points of a warp that stay in registers
+constexpr int kFpsRegPoints = 512;  // points of a warp that stay in registers (16 a thread)
 // Up to this many points one CTA takes them all (0.9 us a choice; 0.3 us in
 // all CTAs from 4,096 points): fewer do not leave room for the exchange in
 // the workspace, which is sized by the points.
@@ -588,13 +590,23 @@ cudaError_t launch_fps(const float* pts, const float* nrm, int64_t n, int32_t k,
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         a.perm = perm;
     }
-    if (a.per_warp <= 32) return fps_launch<1>(a, ctas, s);
-    if (a.per_warp <= 64) return fps_launch<2>(a, ctas, s);
-    if (a.per_warp <= 128) return fps_launch<4>(a, ctas, s);
-    if (a.per_warp <= 256) return fps_launch<8>(a, ctas, s);
-    if (a.per_warp <= 320) return fps_launch<10>(a, ctas, s);
-    if (a.per_warp <= kFpsRegPoints) return fps_launch<16>(a, ctas, s);
-    return fps_launch<0>(a, ctas, s);
+    // Points a thread: one, or the next even number. A slot past the end costs
+    // what a point costs, two of them 5 to 6% of the call (4,096 choices, us:
+    // 400,000 points in 6 / 8 slots 1,459 / 1,541; 700,000 in 10 / 12 / 16
+    // 1,759 / 1,875 / 2,074; 850,000 in 12 / 16 1,864 / 2,063; 1,000,000 in 14 /
+    // 16 2,023 / 2,111).
+    switch (a.per_warp <= 32 ? 1 : 2 * ((a.per_warp + 63) / 64)) {
+    case 1: return fps_launch<1>(a, ctas, s);
+    case 2: return fps_launch<2>(a, ctas, s);
+    case 4: return fps_launch<4>(a, ctas, s);
+    case 6: return fps_launch<6>(a, ctas, s);
+    case 8: return fps_launch<8>(a, ctas, s);
+    case 10: return fps_launch<10>(a, ctas, s);
+    case 12: return fps_launch<12>(a, ctas, s);
+    case 14: return fps_launch<14>(a, ctas, s);
+    case 16: return fps_launch<16>(a, ctas, s);
+    default: return fps_launch<0>(a, ctas, s);  // (more than kFpsRegPoints a warp)
+    }
 }
 
 }  // namespace sop

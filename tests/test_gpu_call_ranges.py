@@ -292,3 +292,35 @@ def test_adjoint_dispatch(sop, orc, R, M, K, S, dtype):
         for got, ref in ((g["env"], w["env"]), (g["maps"][..., :3], w["maps_rgb"]), (g["maps"][..., 3], w["maps_occ"])):
             d = np.abs(got.cpu().numpy() - ref)
             assert np.all(d <= 1e-4 * np.abs(ref) + 2e-5 * np.abs(ref).max() + 1e-12)
+
+
+@pytest.mark.parametrize("n,k,lattice", [
+    (1500, 300, False), (2048, 400, False), (2049, 400, False), (2049, 2049, False),  # one CTA / the least that many share
+    (466_944, 30, False), (466_945, 30, False),      # 6 / 8 points a thread on 152 SMs
+    (778_241, 30, False), (933_889, 30, False), (1_089_537, 30, False),  # 12, 14, 16
+    (4913, 600, True), (110_592, 300, True),         # a lattice: equal keys everywhere
+])
+def test_placement_splits(sop, orc, n, k, lattice):
+    """Probe placement at the edges of its splits, and where nearly every choice
+    is a tie: the indices equal the oracle's, captured in a graph too."""
+    rng = np.random.default_rng(n)
+    if lattice:
+        m = round(n ** (1 / 3))
+        pts = (np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3) / 64).astype(F)
+        pts = pts[rng.permutation(len(pts))]
+    else:
+        pts = rng.standard_normal((n, 3))
+        pts = (pts / np.linalg.norm(pts, axis=1, keepdims=True)).astype(F)
+    d = cuda(pts)
+    want, _ = orc.fps(pts, k, start=n // 2)
+    idx, pos = sop.place_probes(d, k, start=n // 2)
+    assert np.array_equal(idx.cpu().numpy(), want)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        idx, pos = sop.place_probes(d, k, start=n // 2)
+    for _ in range(2):
+        idx.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(idx.cpu().numpy(), want) and np.array_equal(pos.cpu().numpy(), pts[want])
+    sop.device_status()
