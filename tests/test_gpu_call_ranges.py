@@ -324,3 +324,27 @@ def test_placement_splits(sop, orc, n, k, lattice):
         torch.cuda.synchronize()
         assert np.array_equal(idx.cpu().numpy(), want) and np.array_equal(pos.cpu().numpy(), pts[want])
     sop.device_status()
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 1024, 1025, 4096, 4097, 9000])
+def test_bins_of_small_sets(sop, orc, n):
+    """Sets of one Gaussian to a few CTAs' worth, sized so that rays hit whatever
+    their number: the traced maps against the oracle."""
+    rng = np.random.default_rng(n)
+    size = 0.25 * n ** (-1 / 3)
+    s = size * np.exp(rng.uniform(-0.5, 0.5, (n, 3)))
+    q = rng.standard_normal((n, 4))
+    g = dict(mean=rng.uniform(-0.3, 0.3, (n, 3)), scale=s, quat=q / np.linalg.norm(q, axis=1, keepdims=True),
+             opacity=rng.uniform(0.3, 0.9, n), rgb=rng.uniform(0, 1, (n, 3)))
+    g = {k: v.astype(F) for k, v in g.items()}
+    pp, R = np.array([[0.02, -0.05, 0.01], [0.9, 0.1, 0.2], [-0.2, -0.8, 0.5]], F), 8
+    at = sop.make_atlas(cuda(pp), R)
+    sop.bake({k: cuda(v) for k, v in g.items()}, at)
+    sop.device_status()
+    rgb, occ, dep = (t.cpu().numpy() for t in at.interior())
+    o_rgb, o_occ, o_dep, fl, sens = orc.bake(g, pp, R, with_sens=True)
+    decided = (fl & (orc.FLAG_ALPHA_MIN | orc.FLAG_TNEAR | orc.FLAG_TSTOP)) == 0
+    assert decided.mean() > 0.7 and (decided & (o_occ > 0.01)).sum() >= 8
+    assert_close(occ[decided], o_occ[decided], what="O", absolute=sens[..., 3][decided])
+    ok = decided & ((fl & orc.FLAG_ORDER) == 0)
+    assert_close(rgb[ok], o_rgb[ok], what="L_in", absolute=sens[..., :3][ok])
