@@ -424,14 +424,55 @@ def l2_read_peak_gbs(dev):
     return sop.read_bandwidth_gbs(64 << 20, 40, device=dev)
 
 
-def query_demand(K, mode, texel_bytes, M, S, n_normals):
-    """Algorithmic bytes that the SMs must receive from L2/L1 for M points
-    with n_normals distinct normals: per point-direction the 4 texels of each
-    of K probe footprints (RGBO in SHADE mode, O alone in SHADOW mode); per
-    distinct (normal, direction) the 4 environment texels (RGB fp32), since
-    points on one normal share their light directions."""
-    per_texel = texel_bytes if mode == 0 else texel_bytes // 4
-    return K * 4 * per_texel * M * S + 4 * 12 * n_normals * S
+def query_demand(mode, texel_bytes, texels, S, n_normals):
+    """Algorithmic bytes that the SMs must receive from L2/L1: `texels` of the
+    probes' maps (RGBO in SHADE mode, O alone in SHADOW mode) and, per distinct
+    (normal, direction), the 4 environment texels (RGB fp32), since points on
+    one normal share their light directions."""
+    return texels * (texel_bytes if mode == 0 else texel_bytes // 4) + 4 * 12 * n_normals * S
+
+
+def shared_footprints(idx, normals, group=32, most=32):
+    """Probe footprints a light direction that a SHADOW call must read: points
+    of a group (32 next to one another) on one normal, bit for bit, share each
+    of their distinct probes' (up to `most`); any other group reads all of its
+    points'. idx [M, K] int32, normals [M, 3] float32 (tensors)."""
+    import torch
+    M, K = idx.shape
+    total = 0
+    for i0 in range(0, M, group << 14):  # (pieces that fit anywhere)
+        i, n = idx[i0:i0 + (group << 14)], normals[i0:i0 + (group << 14)]
+        pad = -len(i) % group
+        full = i.shape[0] * K
+        if pad:
+            i, n = torch.cat([i, i[-1:].expand(pad, K)]), torch.cat([n, n[-1:].expand(pad, 3)])
+        i, bits = i.reshape(-1, group * K), n.contiguous().view(torch.int32).reshape(-1, group, 3)
+        distinct = 1 + (i.sort(dim=1).values.diff(dim=1) != 0).sum(dim=1)
+        one = (bits == bits[:, :1]).all(dim=2).all(dim=1) & (distinct <= most)
+        total += int(distinct[one].sum()) + full - int(one.sum()) * group * K + (pad * K if bool(one[-1]) else 0)
+    return total
+
+
+def touched_texels(normals, dirs, R):
+    """Texels of an octahedral map (of R x R, with its border) that the bilinear
+    footprints of a point's light directions touch, on average over the normals
+    given. normals [n, 3], dirs [S, 3] (local)."""
+    n = normals.astype(np.float64)
+    n /= np.linalg.norm(n, axis=1, keepdims=True)
+    sg = np.where(n[:, 2] >= 0, 1.0, -1.0)
+    a = -1.0 / (sg + n[:, 2])
+    b = n[:, 0] * n[:, 1] * a
+    t = np.stack([1 + sg * n[:, 0] ** 2 * a, sg * b, -sg * n[:, 0]], axis=1)
+    u = np.stack([b, sg + n[:, 1] ** 2 * a, -n[:, 1]], axis=1)
+    d = dirs.astype(np.float64)
+    w = d[None, :, :1] * t[:, None] + d[None, :, 1:2] * u[:, None] + d[None, :, 2:] * n[:, None]
+    p = w[..., :2] / np.abs(w).sum(-1, keepdims=True)
+    q = (1 - np.abs(p[..., ::-1])) * np.where(p >= 0, 1.0, -1.0)
+    c = np.floor(np.where(w[..., 2:] < 0, q, p) * (0.5 * R) + 0.5 * R - 0.5).astype(int) + 1
+    c = np.clip(c, 0, R)
+    off = c[..., 1] * (R + 2) + c[..., 0]
+    all4 = np.concatenate([off, off + 1, off + R + 2, off + R + 3], axis=1)
+    return float(np.mean([len(np.unique(r)) for r in all4]))
 
 
 def deferred_frame_variant(sop, dev, flush, steps):
@@ -593,6 +634,17 @@ def compose_frame_variant(sop, dev, flush, steps, l2_gbs, hbm_gbs, peak_fp32, ba
                    "pixels (SHADOW), K=8, S=64, 2x4,096 probes at 16x16",
            "points": {q["name"]: q["M"] for q in parts}, "distinct_normals": normals}
     tex_bytes = {"fp32": 16, "bf16": 8, "fp16": 8}
+    touched, shared = {}, {}
+    for q, p in zip(parts, W["parts"]):
+        if q["mode"] == 0:
+            sel = np.random.default_rng(1).choice(q["M"], min(512, q["M"]), replace=False)
+            touched[q["name"]] = touched_texels(p["pts"]["n"][sel], sop.hammersley(S, dev).cpu().numpy(), R)
+        else:
+            _, idx, _ = sop.query_shade(*q["pts"], q["at"], baked.env, K, 1, mode=q["mode"], return_idx=True)
+            shared[q["name"]] = shared_footprints(idx, q["pts"][1])
+            del idx
+    res["footprints"] = {"texels_touched_of_a_map": touched, "shared_probe_footprints_a_point":
+                         {k: round(v / next(q["M"] for q in parts if q["name"] == k), 4) for k, v in shared.items()}}
     for label, st in states.items():
         for _ in range(3):
             for q in st.parts:
@@ -612,9 +664,12 @@ def compose_frame_variant(sop, dev, flush, steps, l2_gbs, hbm_gbs, peak_fp32, ba
                 tp[q["name"]].append(ev[i].elapsed_time(ev[i + 1]))
         ms = float(np.mean(ts))
         pd = st.M * S
-        fl = sum((flop_per_point_dir(K, q["mode"]) - FLOP_DIR_GEOMETRY) * q["M"] * S +
-                 FLOP_DIR_GEOMETRY * normals[q["name"]] * S for q in st.parts)
-        dem = sum(query_demand(K, q["mode"], tex_bytes[label], q["M"], S, normals[q["name"]]) for q in st.parts)
+        fl = sum(((flop_per_point_dir(K, 0) - FLOP_DIR_GEOMETRY) * q["M"] * S if q["mode"] == 0 else
+                  FLOP_SHADOW_FOOTPRINT * shared[q["name"]] * S) + FLOP_DIR_GEOMETRY * normals[q["name"]] * S
+                 for q in st.parts)
+        dem = sum(query_demand(q["mode"], tex_bytes[label], K * q["M"] * min(touched[q["name"]], 4 * S)
+                               if q["mode"] == 0 else 4 * shared[q["name"]] * S, S, normals[q["name"]])
+                  for q in st.parts)
         hbm = 68 * st.M + st.atlas.rgbo.numel() * st.atlas.rgbo.element_size() + st.env.numel() * 4
         t_hbm, t_l2, t_alu = hbm / (hbm_gbs * 1e9), dem / (l2_gbs * 1e9), fl / (peak_fp32 * 1e12)
         bound = max((t_hbm, "hbm"), (t_l2, "l2"), (t_alu, "alu"))
@@ -623,9 +678,9 @@ def compose_frame_variant(sop, dev, flush, steps, l2_gbs, hbm_gbs, peak_fp32, ba
                       "point_dirs_per_s": round(pd / (ms * 1e-3), 1),
                       "roofline": {"kernel": "shade_point_kernel + shadow_warp_kernel and their searches (the frame's "
                                              "two sop_query_shade calls)",
-                                   "note": "l2 counts the texels of every point-direction; points on one normal "
-                                           "share a probe's directions in the SHADOW call, which moves fewer (frac "
-                                           "may exceed 1)",
+                                   "note": "l2 counts each point's touched texels once (SHADE) and each distinct "
+                                           "probe's footprints once per 32 points on one normal (SHADOW); the "
+                                           "nearest-probe search is in none of the three roofs",
                                    "bound": bound[1], "t_hbm_ms": round(t_hbm * 1e3, 4),
                                    "t_l2_ms": round(t_l2 * 1e3, 4), "t_alu_ms": round(t_alu * 1e3, 4),
                                    "frac": round(bound[0] * 1e3 / ms, 4), "l2_demand_bytes": int(dem),
@@ -733,6 +788,8 @@ def depth_precision(sop, W, dev, n_probes=16):
 # the part of flop_per_point_dir that depends only on the normal and the
 # direction: frame rotation, octahedral encode, texel coordinates, environment
 FLOP_DIR_GEOMETRY = 15 + 12 + 10 + 40 + 24 + 8
+# a probe's occlusion at one direction (3 lerps of 3, 1 - O) into three sums
+FLOP_SHADOW_FOOTPRINT = 3 * 3 + 1 + 3 * 2
 
 
 def flop_per_point_dir(K, mode):
