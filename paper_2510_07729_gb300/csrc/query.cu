@@ -304,8 +304,11 @@ __device__ __forceinline__ uint64_t unsearched_bound2(const ProbeGrid& G, const 
 // instructions instead of 10. A cell whose nearest point lies beyond the K-th
 // kept key is not read. 2,051,693 pixels of a ground frame, 4,096 probes,
 // K = 8: 497 -> 405 us (5,290 instructions a warp); an object view of 418,111:
-// 178 -> 155 us. Nine CTAs an SM (56 registers, 24 bytes spilled) instead of
-// eight: the frame's whole call 694 -> 678 us, ten (48, 88 bytes): 680.
+// 178 -> 155 us. K 5 to 8: nine CTAs an SM (56 registers, 24 bytes spilled)
+// instead of eight: the frame's whole call 694 -> 678 us, ten (48, 88 bytes):
+// 680. Up to K 4 eight (64 registers): searches of 2,051,693 ground points 383
+// us with nine, 368 with eight, 377 with ten, 391 unbounded (K 1: 276 / 264 /
+// 273 / 282; 418,111 points of an object 158 / 155 / 160 / 161).
 // ---------------------------------------------------------------------------
 // squared distance along one axis from q to the cell interval [lo, lo + cs)
 __device__ __forceinline__ uint64_t axis_gap2(int32_t q, int64_t lo, int32_t cs)
@@ -403,7 +406,7 @@ __device__ __forceinline__ void knn_search(const ProbeGrid& G, const int32_t q[3
 }
 
 template <int KMAX>
-__global__ void __launch_bounds__(128, KMAX <= 8 ? 9 : 1) knn_kernel(const float* __restrict__ x, const float* __restrict__ nrm, int64_t M,
+__global__ void __launch_bounds__(128, KMAX <= 4 ? 8 : (KMAX <= 8 ? 9 : 1)) knn_kernel(const float* __restrict__ x, const float* __restrict__ nrm, int64_t M,
                                                    int32_t K, int32_t id_bits, uint64_t snap_key, uint64_t r2_key,
                                                    const ProbeGrid* __restrict__ gridp,
                                                    const int32_t* __restrict__ cell_start,
@@ -874,7 +877,7 @@ __device__ __forceinline__ float3 env_lookup(const float4* __restrict__ envq, in
 
 // Bilinear lookup of an octahedral environment (Sec. 4.1) at the octahedral
 // coordinates uv of the direction (the probe maps' mapping: no atan2), from
-// the footprint table of env_oct_quad_kernel.
+// the footprint table that env_oct_footprint wrote.
 __device__ __forceinline__ float3 env_oct_lookup(const float4* __restrict__ envq, int H, float2 uv)
 {
     const float s = uv.x * H - 0.5f, t = uv.y * H - 0.5f;
