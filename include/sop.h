@@ -604,7 +604,9 @@ size_t sop_trace_workspace_bytes(int64_t n_gauss);
  * out [rays][16] float32, device, 16-byte aligned: C.rgb, W, N.xyz, D,
  * A.rgb, R, M, 0, 0, 0 (W = sum T alpha; D / W is the unbiased depth along
  * the ray). ws must hold the grid that sop_bake_bin built for the same g and
- * params (with the same ws_bytes). Asynchronous. */
+ * params (with the same ws_bytes); the call keeps its counters there, and may
+ * replace the binned boxes by the Gaussians' normals: the grid still serves
+ * further traces (sop_bake_trace too), one at a time. Asynchronous. */
 sop_status sop_trace_gbuffer(const sop_gaussians* g, const sop_materials* m, const float* origins,
                              int32_t n_origins, const float* dirs, int64_t n_dirs, const sop_bake_params* params,
                              float* out, void* ws, size_t ws_bytes, void* stream);
