@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(128) adjoint_kernel(const AdjK a)
 // keeps one order whatever points share its CTA (probes by index, texels by
 // place), so a point's gradients are the same on every run.
 // Bound: instruction issue and latency (16 warps an SM, 8,000 instructions a
-// point at S = 128). 418,111 points, K = 8, S = 128: 12.4 -> 7.0 ms.
+// point at S = 128). 418,111 points, K = 8, S = 128: 12.4 -> 6.8 ms.
 // ---------------------------------------------------------------------------
 constexpr int kAdjPts = 8;
 

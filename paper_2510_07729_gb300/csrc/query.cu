@@ -1260,7 +1260,10 @@ __global__ void __launch_bounds__(256, 4) shade_kernel(const ShadeK a, const int
 // (about 10 distinct of 256); a warp with more than kShadowProbes of them, or
 // with several normals, blends per point and direction as shade_kernel does.
 // Bound: the reads of normals, indices and weights, then issue. 2,051,693
-// ground points, K = 8, S = 64, 16-bit atlas: 716 -> 255 us.
+// ground points, K = 8, S = 64, 16-bit atlas: 716 -> 262 us (normals equal bit for
+// bit, as an analytic plane's are; normals of a traced G-buffer differ in their
+// last bits from pixel to pixel: the whole call 1,945 -> 1,739 us with 1e-7 of
+// noise, most of it from the search).
 // ---------------------------------------------------------------------------
 constexpr int kShadowProbes = 32;
 // Whole calls, us (lanes / warp): 16-bit atlas, S 64: 32,768 points 163 / 208,
