@@ -348,3 +348,23 @@ def test_bins_of_small_sets(sop, orc, n):
     assert_close(occ[decided], o_occ[decided], what="O", absolute=sens[..., 3][decided])
     ok = decided & ((fl & orc.FLAG_ORDER) == 0)
     assert_close(rgb[ok], o_rgb[ok], what="L_in", absolute=sens[..., :3][ok])
+
+
+@pytest.mark.parametrize("n", [2000, 20_000])
+def test_bake_replayed_from_a_graph(sop, n):
+    """A bake with default scratch captured in a graph and replayed beside plain
+    bakes of other Gaussians: the plain call's maps, bit for bit."""
+    pp = cuda(np.random.default_rng(2).uniform(-1, 1, (64, 3)).astype(F))
+    g, other = ({k: cuda(v) for k, v in _rods(n, 0.05, 0.01, False, seed).items()} for seed in (5, 6))
+    want, spare, at = (sop.make_atlas(pp, 8) for _ in range(3))
+    sop.bake(g, want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sop.bake(g, at)
+    for _ in range(3):
+        at.rgbo.zero_()
+        sop.bake(other, spare)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(at.rgbo, want.rgbo) and torch.equal(at.depth, want.depth)
